@@ -386,6 +386,7 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
         dt.Bul = h.Bul;
         dt.alpha0 = h.alpha0;
         dt.f = h.f;
+        da.col_c[t] = (h.kind == 0 ? h.f : h.alpha0) / (kH * h.nu0);
         dt.ln_atop = h.kind == 0 ? std::log(h.a_top) : 0.0;
         dt.ln_abot = h.kind == 0 ? std::log(h.a_bot) : 0.0;
     }

@@ -58,6 +58,7 @@ struct DevAtom {
     float muf[RH_MAXMU], wm2f[RH_MAXMU];   // mu and w_mu / 2 for the FP32 sweep
     float imuf[RH_MAXMU];                    // 1/mu
     DevTrans tr[RH_MAXTR];
+    double col_c[RH_MAXTR];       // collisional rates: line f / dE, continuum alpha0 / (h nu0)
     DevTile tile[RH_MAXTILE];
     int16_t order[RH_MAXTILE];               // tile processing order (most expensive first)
     // accumulator -> rate-matrix entry map: A[row][col] += sign * acc
