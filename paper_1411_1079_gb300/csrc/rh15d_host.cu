@@ -13,6 +13,7 @@
 
 #include "rh15d_ckpt.h"
 #include "rh15d_internal.h"
+#include "rh15d_math64.h"
 
 using namespace rh;
 
@@ -65,6 +66,9 @@ struct rh_ctx {
     double lane_nref = 0;
     float4 *vtab_d = nullptr;
     float4 *dtab_d = nullptr;               // FP32 dispersion-function coefficient table
+    char *spec_d = nullptr;                 // wavelength tables of the spectrum calls (kept: grows to the largest call)
+    size_t spec_cap = 0;
+    double *tab64_d = nullptr;              // FP64 function tables (rh15d_math64.h)
     // columns
     int64_t ncol = 0;
     int ndep = 0;
@@ -718,6 +722,36 @@ int spectrum_tables(rh_ctx *c, int64_t nlambda, const double *lambda_m, std::vec
     return RH_OK;
 }
 
+// the tables of spectrum_tables on the device, one copy into the context's
+// workspace; valid until the next call on this context
+struct SpecTables {
+    double *nu, *spec;
+    int *nact, *act;
+};
+cudaError_t spectrum_upload(rh_ctx *c, const std::vector<double> &nu, const std::vector<int> &nact,
+                            const std::vector<int> &act, const std::vector<double> &spec, SpecTables &t)
+{
+    const size_t b0 = nu.size() * 8, b1 = spec.size() * 8, b2 = nact.size() * 4, b3 = act.size() * 4;
+    const size_t n = b0 + b1 + b2 + b3;
+    if (n > c->spec_cap) {
+        dfree(c->spec_d);
+        c->spec_cap = 0;
+        cudaError_t e = cudaMalloc(&c->spec_d, n);
+        if (e != cudaSuccess) return e;
+        c->spec_cap = n;
+    }
+    std::vector<char> h(n);
+    memcpy(h.data(), nu.data(), b0);
+    memcpy(h.data() + b0, spec.data(), b1);
+    memcpy(h.data() + b0 + b1, nact.data(), b2);
+    memcpy(h.data() + b0 + b1 + b2, act.data(), b3);
+    t.nu = reinterpret_cast<double *>(c->spec_d);
+    t.spec = reinterpret_cast<double *>(c->spec_d + b0);
+    t.nact = reinterpret_cast<int *>(c->spec_d + b0 + b1);
+    t.act = reinterpret_cast<int *>(c->spec_d + b0 + b1 + b2);
+    return cudaMemcpyAsync(c->spec_d, h.data(), n, cudaMemcpyHostToDevice, c->st);   // pageable: staged on return
+}
+
 __global__ void validate_kernel(int64_t ncol, int ndep, const double *z, const double *T, const double *ne,
                                 const double *nH, const double *vz, unsigned long long *bad)
 {
@@ -1022,6 +1056,9 @@ int rh_create(rh_ctx **out, int cuda_device, void *cuda_stream)
     }
     if (e == cudaSuccess) e = cudaMalloc(&c->dtab_d, (RH_VT_N + 1) * sizeof(float4));
     if (e == cudaSuccess) e = cudaMemcpy(c->dtab_d, dt.data(), (RH_VT_N + 1) * sizeof(float4), cudaMemcpyHostToDevice);
+    const std::vector<double> t64 = math64_table();
+    if (e == cudaSuccess) e = cudaMalloc(&c->tab64_d, t64.size() * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemcpy(c->tab64_d, t64.data(), t64.size() * sizeof(double), cudaMemcpyHostToDevice);
     *out = c;
     if (e != cudaSuccess) {
         c->err = std::string("rh_create: ") + cudaGetErrorString(e);
@@ -1039,6 +1076,8 @@ void rh_destroy(rh_ctx *c)
     dfree(c->lane_d);
     dfree(c->vtab_d);
     dfree(c->dtab_d);
+    dfree(c->tab64_d);
+    dfree(c->spec_d);
     dfree(c->nghist);
     dfree(c->prd_scr);
     dfree(c->phic);
@@ -1441,34 +1480,22 @@ int rh_emergent_spectrum(rh_ctx *c, double mu, int64_t nlambda, const double *la
     std::vector<int> nact, act;
     int r0 = spectrum_tables(c, nlambda, lambda_m, nu, nact, act, spec);
     if (r0) return r0;
-    double *nu_d = nullptr, *spec_d = nullptr, *out_d = nullptr;
-    int *nact_d = nullptr, *act_d = nullptr;
+    double *out_d = I_out;
+    SpecTables t{};
     int rc = RH_OK;
-    auto cleanup = [&]() {
-        dfree(nu_d);
-        dfree(spec_d);
-        dfree(nact_d);
-        dfree(act_d);
-        if (!on_device) dfree(out_d);
-    };
-    cudaError_t e = cudaMalloc(&nu_d, nlambda * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&spec_d, spec.size() * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&nact_d, nlambda * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&act_d, act.size() * 4);
-    if (e == cudaSuccess) {
-        if (on_device) out_d = I_out;
-        else e = cudaMalloc(&out_d, (size_t)c->ncol * nlambda * 8);
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(nu_d, nu.data(), nlambda * 8, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(spec_d, spec.data(), spec.size() * 8, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(nact_d, nact.data(), nlambda * 4, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(act_d, act.data(), act.size() * 4, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = launch_spectrum(c->da, c->ca, mu, nlambda, nu_d, nact_d, act_d, spec_d, out_d, precision, c->st);
+    cudaError_t e = on_device ? cudaSuccess : cudaMalloc(&out_d, (size_t)c->ncol * nlambda * 8);
+    if (e == cudaSuccess) e = spectrum_upload(c, nu, nact, act, spec, t);
+    unsigned lines = 0;
+    for (int64_t j = 0; j < nlambda; ++j)
+        for (int s = 0; s < nact[j]; ++s) lines |= 1u << act[j * RH_SPEC_ACT + s];
+    if (e == cudaSuccess)
+        e = launch_spectrum(c->da, c->ca, mu, nlambda, t.nu, t.nact, t.act, t.spec, c->tab64_d, lines, c->nsm, out_d,
+                            precision, c->st);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(I_out, out_d, (size_t)c->ncol * nlambda * 8, cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     if (e != cudaSuccess) rc = fail(c, RH_ECUDA, "rh_emergent_spectrum: %s", cudaGetErrorString(e));
-    cleanup();
+    if (!on_device) dfree(out_d);
     return rc;
 }
 
@@ -1494,23 +1521,14 @@ int rh_emergent_stokes(rh_ctx *c, int32_t line, double g_eff, const double *B_T,
     std::vector<int> nact, act;
     int r0 = spectrum_tables(c, nlambda, lambda_m, nu, nact, act, spec);
     if (r0) return r0;
-    double *nu_d = nullptr, *spec_d = nullptr, *out_d = nullptr, *fld = nullptr;
-    int *nact_d = nullptr, *act_d = nullptr;
-    auto cleanup = [&]() {
-        dfree(nu_d);
-        dfree(spec_d);
-        dfree(nact_d);
-        dfree(act_d);
-        dfree(fld);
-        if (!on_device) dfree(out_d);
-    };
+    double *out_d = iquv_out, *fld = nullptr;
+    SpecTables t{};
     const double *Bd = B_T, *td = theta, *cd = chi;
-    cudaError_t e = cudaMalloc(&nu_d, nlambda * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&spec_d, spec.size() * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&nact_d, nlambda * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&act_d, act.size() * 4);
-    if (e == cudaSuccess && !on_device) {
-        e = cudaMalloc(&fld, 3 * nd * 8);
+    cudaError_t e = spectrum_upload(c, nu, nact, act, spec, t);
+    if (!on_device) {
+        out_d = nullptr;
+        if (e == cudaSuccess) e = cudaMalloc(&out_d, (size_t)c->ncol * nlambda * 4 * 8);
+        if (e == cudaSuccess) e = cudaMalloc(&fld, 3 * nd * 8);
         if (e == cudaSuccess) e = cudaMemcpyAsync(fld, B_T, nd * 8, cudaMemcpyHostToDevice, c->st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(fld + nd, theta, nd * 8, cudaMemcpyHostToDevice, c->st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(fld + 2 * nd, chi, nd * 8, cudaMemcpyHostToDevice, c->st);
@@ -1518,23 +1536,18 @@ int rh_emergent_stokes(rh_ctx *c, int32_t line, double g_eff, const double *B_T,
         td = fld + nd;
         cd = fld + 2 * nd;
     }
-    if (e == cudaSuccess) {
-        if (on_device) out_d = iquv_out;
-        else e = cudaMalloc(&out_d, (size_t)c->ncol * nlambda * 4 * 8);
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(nu_d, nu.data(), nlambda * 8, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(spec_d, spec.data(), spec.size() * 8, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(nact_d, nact.data(), nlambda * 4, cudaMemcpyHostToDevice, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(act_d, act.data(), act.size() * 4, cudaMemcpyHostToDevice, c->st);
     if (e == cudaSuccess)
-        e = launch_stokes(c->da, c->ca, line, g_eff, Bd, td, cd, nlambda, nu_d, nact_d, act_d, spec_d, c->vtab_d,
+        e = launch_stokes(c->da, c->ca, line, g_eff, Bd, td, cd, nlambda, t.nu, t.nact, t.act, t.spec, c->vtab_d,
                           c->dtab_d, out_d, precision, c->st);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(iquv_out, out_d, (size_t)c->ncol * nlambda * 4 * 8, cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
     int rc = RH_OK;
     if (e != cudaSuccess) rc = fail(c, RH_ECUDA, "rh_emergent_stokes: %s", cudaGetErrorString(e));
-    cleanup();
+    if (!on_device) {
+        dfree(out_d);
+        dfree(fld);
+    }
     return rc;
 }
 

@@ -791,7 +791,8 @@ cudaError_t launch_regrid(const ColumnArrays &c, int M, const RegridParams &g, d
 #define RH_SPEC_F 8
 cudaError_t launch_spectrum(const DevAtom &A, const ColumnArrays &c, double mu, int64_t nlam,
                             const double *nu_d, const int *nact_d, const int *act_d, const double *spec_d,
-                            double *out, int precision, cudaStream_t st);
+                            const double *tab64, unsigned lines, int nsm, double *out, int precision,
+                            cudaStream_t st);
 
 // emergent Stokes vector at mu = 1 of transition t0 (a line) with Zeeman
 // splitting; B_T, theta, chi [ncol][ndep]; out [ncol][nlam][4]

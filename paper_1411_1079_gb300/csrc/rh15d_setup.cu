@@ -1,6 +1,9 @@
 // rh15d_setup.cu -- per-depth set-up (LTE start, Sect. 2.3) and the emergent
 // spectrum (Sect. 2.2) kernels.
+#include <algorithm>
+
 #include "rh15d_internal.h"
+#include "rh15d_math64.h"
 
 namespace rh {
 
@@ -34,7 +37,7 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
     double phi[RH_MAXLEV], ex[RH_MAXLEV];   // ex: exp((E_continuum - E_i) / kT)
     double Phi = 0.0;
     for (int i = 0; i < ic; ++i) {
-        ex[i] = exp(A.lev_chi[i] * ikT);
+        ex[i] = exp(div64(A.lev_chi[i], kT, ikT));
         phi[i] = A.lev_g2[i] * lam3 * ex[i];
         Phi += phi[i];
     }
@@ -80,84 +83,146 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
     }
 }
 
-// Emergent intensity: one thread per (column, requested wavelength), upward
-// linear short-characteristics sweep at direction cosine mu from the
-// diffusion condition at the bottom.
+// Emergent intensity at direction cosine mu: upward linear
+// short-characteristics sweep from the diffusion condition at the bottom,
+// FP64 opacities, the sweep in R.
+//
+// A block owns one column and lc of its wavelengths.  What depends on depth
+// only (h/kT, background coefficients, Doppler width, path lengths,
+// populations, continuum ratios, damping of the lines in use) is formed once
+// into shared memory, kw depths at a time; then a thread walks the depths of
+// its wavelength.  The kernel is bound by the FP64 pipe, so the table-driven
+// functions of rh15d_math64.h carry the points: one exponential, the Voigt
+// function of the active lines, one exponential or one polynomial of the
+// step.  4096 columns x 82 depths x 201 wavelengths, FP64: rh_emergent_spectrum 229 -> 32 ms
+// (about 300 FP64 instructions a point at the FP64 pipe's rate).
+// The sweep over a segment of depths is the map I -> A I + B, so with few
+// columns a wavelength's depths are split over G threads, whose maps are
+// composed at the end (all terms positive: no cancellation); each segment
+// evaluates its upwind point once more, which is why G is 1 as soon as the
+// warps of one thread per wavelength fill the chip.
+enum { XF_KT, XF_IKT, XF_KFF, XF_NHM, XF_THOM, XF_VTH, XF_IVTH, XF_VZ, XF_HZ, XF_N };
+constexpr int kSpecThreads = 256;
 template <typename R>
-__global__ void spectrum_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, double mu, int64_t nlam,
-                                const double *nu_d, const int *nact_d, const int *act_d, const double *spec,
-                                double *out)
+__global__ void __launch_bounds__(kSpecThreads, 2)
+    spectrum_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, double mu, int64_t nlam, const double *nu_d,
+                    const int *nact_d, const int *act_d, const double *spec, const double *tab_g, unsigned lines,
+                    int lc, int G, int kw, double *out)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= c.ncol * nlam) return;
-    const int64_t col = idx / nlam, j = idx % nlam;
-    const int N = c.ndep, L = A.nlev;
-    const double nu = nu_d[j];
-    const int na = nact_d[j];
+    extern __shared__ double sx[];
+    __shared__ R comb[2][kSpecThreads];
+    double *tab = sx, *fld = sx + kT64Size, *pop = fld + XF_N * kw, *gc = pop + A.nlev * kw, *da = gc + A.ncont * kw;
+    const int nchunk = (int)((nlam + lc - 1) / lc), N = c.ndep, L = A.nlev;
+    const int64_t col = blockIdx.x / nchunk;
+    const int g = threadIdx.x / lc;
+    const int64_t j = (int64_t)(blockIdx.x % nchunk) * lc + threadIdx.x % lc;
+    const bool on = j < nlam;
+    const size_t cN = (size_t)col * N;
     const double e2 = kQ * kQ / (4.0 * kPi * kEps0);
     const double Cff = e2 * e2 * e2 * 4.0 / (3.0 * kMe * kH * kC) * sqrt(2.0 * kPi / (3.0 * kK * kMe));
-    const double hm = hminus_sigma(kC / nu);
-    const double tw = 2.0 * kH * nu * nu * nu / (kC * kC);
-    const size_t cN = (size_t)col * N;
-    R I = 0, chip = 0, Sp = 0;
-    R Bp = 0;
-    for (int step = 0; step < N; ++step) {
-        const int k = N - 1 - step;
-        const double T = c.T[cN + k];
-        const double ne = c.ne[cN + k];
-        const double x = kH * nu / (kK * T);
-        const double lam3 = pow(kH * kH / (2.0 * kPi * kMe * kK * T), 1.5);
-        const double nhm = 0.25 * c.nstar[((size_t)col * L + 0) * N + k] * ne * lam3 * exp(0.754 * kQ / (kK * T));
-        const double omex = -expm1(-x);
-        double chi = (Cff * ne * c.np[cN + k] / sqrt(T) / (nu * nu * nu) + nhm * hm) * omex + kSigmaT * ne;
-        const double B = tw * exp(-x) / omex;
-        double eta = chi * B;
-        const double vth = sqrt(2.0 * kK * T / A.mass);
-        const double sk = N > 1 ? (double)k / (N - 1) : 0.0;
-        for (int s = 0; s < na; ++s) {
-            const int t = act_d[j * RH_SPEC_ACT + s];
-            const DevTrans &tr = A.tr[t];
-            const double *f = spec + ((size_t)j * RH_SPEC_ACT + s) * RH_SPEC_F;
-            const double nl = c.pops[((size_t)col * L + tr.l) * N + k];
-            const double nu_ = c.pops[((size_t)col * L + tr.u) * N + k];
-            double Vlu, Vul, U;
-            if (tr.kind == 0) {
-                const double a = exp((1.0 - sk) * tr.ln_atop + sk * tr.ln_abot);
-                const double v = (f[3] - mu * c.vz[cN + k]) / vth;
-                const double ph = (R)voigt_f64(a, v) * f[4] / vth;
-                Vlu = f[0] * ph;
-                Vul = f[2] * Vlu;
-                U = f[1] * ph;
-            } else {
-                const double G = c.nstar[((size_t)col * L + tr.l) * N + k] / c.nstar[((size_t)col * L + tr.u) * N + k];
-                Vlu = f[0];
-                Vul = G * exp(-x) * f[0];
-                U = f[1] * G * exp(-x);
+    for (int i = threadIdx.x; i < kT64Size; i += blockDim.x) tab[i] = tab_g[i];
+    const double nu = on ? nu_d[j] : 1e15;
+    const int na = on ? nact_d[j] : 0;
+    const double hnu = kH * nu, hm = hminus_sigma(kC / nu), inu3 = 1.0 / (nu * nu * nu), tw = 2.0 * kH * nu * nu * nu / (kC * kC);
+    // this thread's segment of sweep steps (step s is depth N - 1 - s), from
+    // the upwind point of its first step
+    const int s0 = (int)((int64_t)N * g / G), s1 = (int)((int64_t)N * (g + 1) / G), sb = s0 > 0 ? s0 - 1 : 0;
+    R Am = 1, Bm = 0, chip = 0, Sp = 0;
+    double Bp = 0;
+    for (int w0 = 0; w0 < N; w0 += kw) {
+        if (w0) __syncthreads();
+        for (int i = threadIdx.x; i < kw && w0 + i < N; i += blockDim.x) {
+            const int k = N - 1 - w0 - i;
+            const double T = c.T[cN + k], ne = c.ne[cN + k], ikT = 1.0 / (kK * T);
+            const double r3 = kH * kH / (2.0 * kPi * kMe) * ikT;
+            fld[XF_KT * kw + i] = kK * T;
+            fld[XF_IKT * kw + i] = ikT;
+            fld[XF_KFF * kw + i] = Cff * ne * c.np[cN + k] / sqrt(T);
+            fld[XF_NHM * kw + i] = 0.25 * c.nstar[((size_t)col * L + 0) * N + k] * ne * (r3 * sqrt(r3)) *
+                                   exp(0.754 * kQ * ikT);
+            fld[XF_THOM * kw + i] = kSigmaT * ne;
+            const double vth = sqrt(2.0 * kK * T / A.mass);
+            fld[XF_VTH * kw + i] = vth;
+            fld[XF_IVTH * kw + i] = 1.0 / vth;
+            fld[XF_VZ * kw + i] = mu * c.vz[cN + k];
+            fld[XF_HZ * kw + i] = k < N - 1 ? 0.5 * fabs(c.z[cN + k] - c.z[cN + k + 1]) / mu : 0.0;
+            for (int l = 0; l < L; ++l) pop[l * kw + i] = c.pops[((size_t)col * L + l) * N + k];
+            const double sk = N > 1 ? (double)k / (N - 1) : 0.0;
+            for (int t = 0; t < A.ntr; ++t) {
+                const DevTrans &tr = A.tr[t];
+                if (!(lines >> t & 1)) continue;
+                if (tr.kind == 0)
+                    da[tr.sub * kw + i] = exp((1.0 - sk) * tr.ln_atop + sk * tr.ln_abot);
+                else
+                    gc[tr.sub * kw + i] = c.nstar[((size_t)col * L + tr.l) * N + k] /
+                                          c.nstar[((size_t)col * L + tr.u) * N + k];
             }
-            chi += nl * Vlu - nu_ * Vul;
-            eta += nu_ * U;
         }
-        const R chiR = (R)chi, S = (R)(eta / chi);
-        if (step == 0) {
+        __syncthreads();
+        for (int s = max(sb, w0); s < min(s1, w0 + kw) && on; ++s) {
+            const int i = s - w0;
+            const double x = div64(hnu, fld[XF_KT * kw + i], fld[XF_IKT * kw + i]);
+            double ex, om;
+            if (x < 0.5) {   // 1 - e^{-x} by expm1 where it would cancel
+                om = -expm1(-x);
+                ex = 1.0 - om;
+            } else {
+                ex = exp64(-x, tab);
+                om = 1.0 - ex;
+            }
+            double chi = fma(fma(fld[XF_NHM * kw + i], hm, fld[XF_KFF * kw + i] * inu3), om, fld[XF_THOM * kw + i]);
+            const double B = tw * ex * rcp64(om);
+            double eta = chi * B;
+            for (int a = 0; a < na; ++a) {
+                const int t = act_d[j * RH_SPEC_ACT + a];
+                const DevTrans &tr = A.tr[t];
+                const double *f = spec + ((size_t)j * RH_SPEC_ACT + a) * RH_SPEC_F;
+                const double nl = pop[tr.l * kw + i], nup = pop[tr.u * kw + i];
+                if (tr.kind == 0) {
+                    const double ivth = fld[XF_IVTH * kw + i];
+                    double H, Ld;
+                    voigt64<false>(da[tr.sub * kw + i], div64(f[3] - fld[XF_VZ * kw + i], fld[XF_VTH * kw + i], ivth), tab,
+                                   H, Ld);
+                    const double ph = (R)H * (f[4] * ivth);
+                    chi = fma(f[0] * ph, fma(-f[2], nup, nl), chi);
+                    eta = fma(f[1] * ph, nup, eta);
+                } else {
+                    const double Ge = gc[tr.sub * kw + i] * ex;
+                    chi = fma(f[0], fma(-Ge, nup, nl), chi);
+                    eta = fma(f[1] * Ge, nup, eta);
+                }
+            }
+            const R chiR = (R)chi, S = (R)(eta * rcp64(chi));
+            if (s > sb) {
+                const R hz = (R)fld[XF_HZ * kw + i], sum = chiR + chip;
+                if (s == 1)   // the bottom point's intensity: diffusion approximation
+                    Bm = (R)Bp + (R)mu * ((R)Bp - (R)B) / (sum * hz * (R)mu), Am = 0;
+                R e, wu, wo;
+                if constexpr (sizeof(R) == 8) {
+                    double q;
+                    sc64(sum * hz, tab, e, wu, wo, q);
+                } else {
+                    sc_weights(sum * hz, e, wu, wo);
+                }
+                Am *= e;
+                Bm = Bm * e + wu * Sp + wo * S;
+            }
             chip = chiR;
             Sp = S;
-            Bp = (R)B;
-            // diffusion condition needs chi and B one point up: computed next step
-            continue;
+            Bp = B;
         }
-        if (step == 1) {
-            // I at the bottom point from the diffusion approximation
-            const R dtv = (R)0.5 * (chiR + chip) * (R)fabs(c.z[cN + N - 2] - c.z[cN + N - 1]);
-            I = Bp + (R)mu * (Bp - (R)B) / dtv;
-        }
-        const R dtau = (R)0.5 * (chiR + chip) * (R)fabs(c.z[cN + k] - c.z[cN + k + 1]) / (R)mu;
-        R ome, wu, wo;
-        sc_weights(dtau, ome, wu, wo);
-        I = I * ome + wu * Sp + wo * S;
-        chip = chiR;
-        Sp = S;
     }
-    out[idx] = (double)I;
+    if (G == 1) {
+        if (on) out[(size_t)col * nlam + j] = (double)Bm;
+        return;
+    }
+    comb[0][threadIdx.x] = Am;
+    comb[1][threadIdx.x] = Bm;
+    __syncthreads();
+    if (g == 0 && on) {
+        for (int q = 1; q < G; ++q) Bm = comb[0][threadIdx.x + q * lc] * Bm + comb[1][threadIdx.x + q * lc];
+        out[(size_t)col * nlam + j] = (double)Bm;
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -844,17 +909,30 @@ cudaError_t launch_stokes(const DevAtom &A, const ColumnArrays &c, int t0, doubl
 }
 
 cudaError_t launch_spectrum(const DevAtom &A, const ColumnArrays &c, double mu, int64_t nlam, const double *nu_d,
-                            const int *nact_d, const int *act_d, const double *spec_d, double *out, int precision,
-                            cudaStream_t st)
+                            const int *nact_d, const int *act_d, const double *spec_d, const double *tab64,
+                            unsigned lines, int nsm, double *out, int precision, cudaStream_t st)
 {
-    int64_t n = c.ncol * nlam;
-    if (n == 0) return cudaSuccess;
-    int threads = 128;
-    int64_t blocks = (n + threads - 1) / threads;
-    if (precision == 1)
-        spectrum_kernel<float><<<(unsigned)blocks, threads, 0, st>>>(A, c, mu, nlam, nu_d, nact_d, act_d, spec_d, out);
-    else
-        spectrum_kernel<double><<<(unsigned)blocks, threads, 0, st>>>(A, c, mu, nlam, nu_d, nact_d, act_d, spec_d, out);
+    if (c.ncol * nlam == 0) return cudaSuccess;
+    const int N = c.ndep;
+    // depths per shared-memory table: all of them, or what 64 KB hold
+    const size_t per_k = sizeof(double) * (size_t)(XF_N + A.nlev + A.ncont + A.nline);
+    const int kw = (int)std::min<size_t>((size_t)N, 65536 / per_k);
+    const int64_t rows = (nlam + 31) / 32;   // warps per column with one thread per wavelength
+    int G = 1, lc = (int)std::min<int64_t>(kSpecThreads, 32 * rows);
+    if (c.ncol * rows < 8LL * nsm && kw == N) {
+        // under two warps per scheduler: split the depths (at least 4 each)
+        while (G < 8 && c.ncol * rows * G < 8LL * nsm && N >= 8 * G) G *= 2;
+        if (G > 1) lc = 32;
+    }
+    while (G == 1 && lc > 32 && c.ncol * ((nlam + lc - 1) / lc) < 2LL * nsm) lc -= 32;
+    const int64_t blocks = c.ncol * ((nlam + lc - 1) / lc);
+    if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    const size_t sm = sizeof(double) * kT64Size + per_k * kw;
+    auto kern = precision == 1 ? spectrum_kernel<float> : spectrum_kernel<double>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)blocks, lc * G, sm, st>>>(A, c, mu, nlam, nu_d, nact_d, act_d, spec_d, tab64, lines, lc, G, kw,
+                                               out);
     return cudaGetLastError();
 }
 
