@@ -1538,7 +1538,7 @@ int rh_emergent_stokes(rh_ctx *c, int32_t line, double g_eff, const double *B_T,
     }
     if (e == cudaSuccess)
         e = launch_stokes(c->da, c->ca, line, g_eff, Bd, td, cd, nlambda, t.nu, t.nact, t.act, t.spec, c->vtab_d,
-                          c->dtab_d, out_d, precision, c->st);
+                          c->dtab_d, c->tab64_d, out_d, precision, c->st);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(iquv_out, out_d, (size_t)c->ncol * nlambda * 4 * 8, cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);

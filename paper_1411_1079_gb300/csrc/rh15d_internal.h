@@ -798,8 +798,8 @@ cudaError_t launch_spectrum(const DevAtom &A, const ColumnArrays &c, double mu, 
 // splitting; B_T, theta, chi [ncol][ndep]; out [ncol][nlam][4]
 cudaError_t launch_stokes(const DevAtom &A, const ColumnArrays &c, int t0, double geff, const double *B_T,
                           const double *theta, const double *chi, int64_t nlam, const double *nu_d, const int *nact_d,
-                          const int *act_d, const double *spec_d, const float4 *vtab, const float4 *dtab, double *out,
-                          int precision, cudaStream_t st);
+                          const int *act_d, const double *spec_d, const float4 *vtab, const float4 *dtab,
+                          const double *tab64, double *out, int precision, cudaStream_t st);
 
 // learned initial guess (rh15d_mlp.cu)
 struct Mlp;

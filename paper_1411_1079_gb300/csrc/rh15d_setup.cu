@@ -391,18 +391,17 @@ __global__ void start_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, 
 // K' = K/eI - 1 and S the emission / eI; 4 x 4 solve with partial pivoting.
 // Bottom: I = B + dB/dtau (diffusion), Q = U = V = 0.
 template <typename R>
-__device__ __forceinline__ void zeeman_profiles(R a, R v, R vB, const float4 *vtab, const float4 *dtab, R *H, R *L);
+__device__ __forceinline__ void zeeman_profiles(R a, R v, R vB, const float4 *vtab, const float4 *dtab,
+                                                const double *tab64, R *H, R *L);
 template <>
-__device__ __forceinline__ void zeeman_profiles<double>(double a, double v, double vB, const float4 *,
-                                                        const float4 *, double *H, double *L)
+__device__ __forceinline__ void zeeman_profiles<double>(double a, double v, double vB, const float4 *, const float4 *,
+                                                        const double *tab64, double *H, double *L)
 {
-    faddeeva_f64(a, v - vB, H[0], L[0]);
-    faddeeva_f64(a, v, H[1], L[1]);
-    faddeeva_f64(a, v + vB, H[2], L[2]);
+    for (int i = 0; i < 3; ++i) voigt64<true>(a, v + (i - 1) * vB, tab64, H[i], L[i]);
 }
 template <>
 __device__ __forceinline__ void zeeman_profiles<float>(float a, float v, float vB, const float4 *vtab,
-                                                       const float4 *dtab, float *H, float *L)
+                                                       const float4 *dtab, const double *, float *H, float *L)
 {
     const float vs[3] = {v - vB, v, v + vB};
 #pragma unroll
@@ -412,73 +411,39 @@ __device__ __forceinline__ void zeeman_profiles<float>(float a, float v, float v
     }
 }
 
+// One DELO-linear step: (1 + w_o K'_o) I_o = b in closed form.  K' acts on (I,
+// v = (Q, U, V)) as I' = e.v, v' = e I + v x r with e = (eQ, eU, eV), r = (rQ,
+// rU, rV) (over eI).  With w_o in e and r, v + v x r = w has the solution
+// M(w) = [w + r (r.w) - w x r] / (1 + r^2), so v = M(w - e I) = M(w) - I M(e)
+// and I = (b_0 - e.M(w)) / (1 - e.M(e)), e.M(e) = [e^2 + (e.r)^2] / (1 + r^2) <=
+// e^2 <= w_o^2 < 1.  Some 70 operations and two reciprocals for the 4x4
+// elimination with partial pivoting (about 250 with its selects).
 template <typename R>
-__device__ void delo_step(R ex, R wu, R wo, const R *Ku, const R *Ko, const R *Su, const R *So, R *I)
+__device__ __forceinline__ void delo_step(R ex, R wu, R wo, const R *Ku, const R *Ko, const R *Su, const R *So, R *I)
 {
-    // K'(k) from (eQ, eU, eV, rQ, rU, rV)/eI
-    auto kp = [](const R *k, R M[4][4]) {
-        M[0][0] = 0; M[0][1] = k[0]; M[0][2] = k[1]; M[0][3] = k[2];
-        M[1][0] = k[0]; M[1][1] = 0; M[1][2] = k[5]; M[1][3] = -k[4];
-        M[2][0] = k[1]; M[2][1] = -k[5]; M[2][2] = 0; M[2][3] = k[3];
-        M[3][0] = k[2]; M[3][1] = k[4]; M[3][2] = -k[3]; M[3][3] = 0;
-    };
-    R Mu[4][4], A[4][4], b[4];
-    kp(Ku, Mu);
-    kp(Ko, A);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        R kI = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) kI += Mu[i][j] * I[j];
-        b[i] = ex * I[i] + wu * (Su[i] - kI) + wo * So[i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) A[i][j] = (i == j ? (R)1 : (R)0) + wo * A[i][j];
-    }
-    // Gaussian elimination with partial pivoting (fixed size, unrolled)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        int piv = c;
-#pragma unroll
-        for (int r = c + 1; r < 4; ++r)
-            if (fabs(A[r][c]) > fabs(A[piv][c])) piv = r;
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-            if (r == piv && piv != c) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    R tq = A[c][q];
-                    A[c][q] = A[r][q];
-                    A[r][q] = tq;
-                }
-                R tb = b[c];
-                b[c] = b[r];
-                b[r] = tb;
-            }
-        const R ip = (R)1 / A[c][c];
-#pragma unroll
-        for (int r = c + 1; r < 4; ++r) {
-            const R f = A[r][c] * ip;
-#pragma unroll
-            for (int q = c; q < 4; ++q) A[r][q] -= f * A[c][q];
-            b[r] -= f * b[c];
-        }
-    }
-#pragma unroll
-    for (int c = 3; c >= 0; --c) {
-        R s = b[c];
-#pragma unroll
-        for (int q = c + 1; q < 4; ++q) s -= A[c][q] * b[q];
-        b[c] = s / A[c][c];
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) I[i] = b[i];
+    R b[4];
+    b[0] = ex * I[0] + wu * (Su[0] - (Ku[0] * I[1] + Ku[1] * I[2] + Ku[2] * I[3])) + wo * So[0];
+    b[1] = ex * I[1] + wu * (Su[1] - (Ku[0] * I[0] + Ku[5] * I[2] - Ku[4] * I[3])) + wo * So[1];
+    b[2] = ex * I[2] + wu * (Su[2] - (Ku[1] * I[0] - Ku[5] * I[1] + Ku[3] * I[3])) + wo * So[2];
+    b[3] = ex * I[3] + wu * (Su[3] - (Ku[2] * I[0] + Ku[4] * I[1] - Ku[3] * I[2])) + wo * So[3];
+    const R e0 = wo * Ko[0], e1 = wo * Ko[1], e2 = wo * Ko[2], r0 = wo * Ko[3], r1 = wo * Ko[4], r2 = wo * Ko[5];
+    const R i1 = (R)1 / ((R)1 + r0 * r0 + r1 * r1 + r2 * r2);
+    const R dw = r0 * b[1] + r1 * b[2] + r2 * b[3], de = r0 * e0 + r1 * e1 + r2 * e2;
+    const R q0 = (b[1] + r0 * dw - (b[2] * r2 - b[3] * r1)) * i1, q1 = (b[2] + r1 * dw - (b[3] * r0 - b[1] * r2)) * i1,
+            q2 = (b[3] + r2 * dw - (b[1] * r1 - b[2] * r0)) * i1;
+    const R p0 = (e0 + r0 * de - (e1 * r2 - e2 * r1)) * i1, p1 = (e1 + r1 * de - (e2 * r0 - e0 * r2)) * i1,
+            p2 = (e2 + r2 * de - (e0 * r1 - e1 * r0)) * i1;
+    I[0] = (b[0] - (e0 * q0 + e1 * q1 + e2 * q2)) / ((R)1 - (e0 * e0 + e1 * e1 + e2 * e2 + de * de) * i1);
+    I[1] = q0 - I[0] * p0;
+    I[2] = q1 - I[0] * p1;
+    I[3] = q2 - I[0] * p2;
 }
 
 template <typename R>
 __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, int t0, double geff, const double *Bf,
                               const double *thf, const double *azf, int64_t nlam, const double *nu_d,
                               const int *nact_d, const int *act_d, const double *spec, const float4 *vtab_g,
-                              const float4 *dtab_g, double *out)
+                              const float4 *dtab_g, const double *tab64, double *out)
 {
     __shared__ float4 tabs[sizeof(R) == 4 ? 2 * (RH_VT_N + 1) : 1];
     const float4 *vtab = tabs, *dtab = tabs + (RH_VT_N + 1);
@@ -509,7 +474,7 @@ __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c,
         const double T = c.T[cN + k];
         const double ne = c.ne[cN + k];
         const double x = kH * nu / (kK * T);
-        const double lam3 = pow(kH * kH / (2.0 * kPi * kMe * kK * T), 1.5);
+        const double r3 = kH * kH / (2.0 * kPi * kMe * kK * T), lam3 = r3 * sqrt(r3);
         const double nhm = 0.25 * c.nstar[((size_t)col * L + 0) * N + k] * ne * lam3 * exp(0.754 * kQ / (kK * T));
         const double omex = -expm1(-x);
         double chi = (Cff * ne * c.np[cN + k] / sqrt(T) / (nu * nu * nu) + nhm * hm) * omex + kSigmaT * ne;
@@ -528,7 +493,9 @@ __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c,
             if (tr.kind == 0) {
                 const double a = exp((1.0 - sk) * tr.ln_atop + sk * tr.ln_abot);
                 const double v = (f[3] - c.vz[cN + k]) / vth;
-                const double ph = voigt_f64(a, v) * f[4] / vth;
+                double H1, L1;
+                voigt64<false>(a, v, tab64, H1, L1);
+                const double ph = H1 * f[4] / vth;
                 Vlu = f[0] * ph;
                 Vul = f[2] * Vlu;
                 U = f[1] * ph;
@@ -551,7 +518,7 @@ __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c,
         const R v = (R)(kC * ((nu - tr0.nu0) / tr0.nu0) / vth - c.vz[cN + k] / vth);
         const R vB = (R)(nuB * Bf[cN + k] / dnuD);
         R Hz[3], Lz[3];
-        zeeman_profiles<R>((R)a0, v, vB, vtab, dtab, Hz, Lz);
+        zeeman_profiles<R>((R)a0, v, vB, vtab, dtab, tab64, Hz, Lz);
         const double th = thf[cN + k], az = azf[cN + k];
         const R s2 = (R)(sin(th) * sin(th)), ct = (R)cos(th), c2 = (R)cos(2.0 * az), sn2 = (R)sin(2.0 * az);
         const R hk = (R)(0.5 * kl);
@@ -581,7 +548,12 @@ __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c,
             }
             const R dtau = (R)0.5 * (eI + eIu) * (R)fabs(c.z[cN + k] - c.z[cN + k + 1]);
             R ome, wu, wo;
-            sc_weights(dtau, ome, wu, wo);
+            if constexpr (sizeof(R) == 8) {
+                double omwo;
+                sc64(dtau, tab64, ome, wu, wo, omwo);
+            } else {
+                sc_weights(dtau, ome, wu, wo);
+            }
             delo_step<R>(ome, wu, wo, Ku, Ko, Su, So, I);
             eIu = eI;
         }
@@ -602,13 +574,18 @@ __global__ void stokes_kernel(const __grid_constant__ DevAtom A, ColumnArrays c,
 // source function, damping, Zeeman splitting and field geometry -- are formed
 // once per depth in FP64 and stored in shared memory in FP32; then every
 // thread sweeps its wavelengths with FP32 opacities, profiles and the same
-// DELO-linear step as stokes_kernel.  Layout of the shared arrays: kSF fields
+// DELO-linear step as stokes_kernel; the other transitions' constants of a
+// wavelength are converted to FP32 once, before its sweep (in the sweep their
+// FP64 products kept the FP64 pipe busy at every depth).  2048 columns x 128
+// depths x 400 wavelengths: 5.2 -> 2.5 ms with the
+// closed-form step.  Layout of the shared arrays: kSF fields
 // [field][N], then the populations [L][N] and continuum ratios [ncont][N].
 constexpr double kStokesNref = 1e20;
 constexpr int kSF = 16;
+constexpr int kStokesThreads = 224;
 enum { SF_HKT, SF_KFF, SF_NHM, SF_THOM, SF_IVTH, SF_VZ, SF_DZ, SF_SK, SF_KL, SF_SL, SF_A0, SF_VB, SF_S2, SF_CT, SF_C2,
        SF_SN2 };
-__global__ void __launch_bounds__(128) stokes32_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, int t0,
+__global__ void __launch_bounds__(kStokesThreads) stokes32_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, int t0,
                                                        double geff, const double *Bf, const double *thf,
                                                        const double *azf, int64_t nlam, const double *nu_d,
                                                        const int *nact_d, const int *act_d, const double *spec,
@@ -677,38 +654,48 @@ __global__ void __launch_bounds__(128) stokes32_kernel(const __grid_constant__ D
             const float nu3s = (float)(kNuRef3 / (nud * nud * nud));
             const float q0 = (float)(kC * ((nud - tr0.nu0) / tr0.nu0));
             const float hr = (float)(nud / tr0.nu0);             // h4(nu) / h4(nu0)
+            // lines: f0, f1 (A), g-ratio, Doppler offset, norm; continua: alpha, emission
+            float cf[RH_SPEC_ACT][5];
+            for (int a = 0; a < na; ++a) {
+                const double *f = spec + ((size_t)j * RH_SPEC_ACT + a) * RH_SPEC_F;
+                const bool line = A.tr[act_d[j * RH_SPEC_ACT + a]].kind == 0;
+                cf[a][0] = (float)(line ? f[0] : f[0] * kStokesNref);
+                cf[a][1] = (float)(line ? f[1] : f[1] * kStokesNref);
+                cf[a][2] = (float)f[2];
+                cf[a][3] = (float)f[3];
+                cf[a][4] = (float)(f[4] * kStokesNref);
+            }
             float I[4] = {0, 0, 0, 0}, Ku[6], Su[4], eIu = 0, Bu = 0;
             for (int step = 0; step < N; ++step) {
                 const int k = N - 1 - step;
                 const float x = nu * sf[SF_HKT * N + k];
                 const float ex = __expf(-x), omex = 1.0f - ex;
                 float chi = (sf[SF_KFF * N + k] * nu3s + sf[SF_NHM * N + k] * hm) * omex + sf[SF_THOM * N + k];
-                const float B = tw * ex / omex;
+                const float B = tw * ex * rcp_f32(omex);
                 float eta = chi * B;
                 const float ivth = sf[SF_IVTH * N + k], vz = sf[SF_VZ * N + k], sk = sf[SF_SK * N + k];
                 for (int s2i = 0; s2i < na; ++s2i) {
                     const int t = act_d[j * RH_SPEC_ACT + s2i];
                     if (t == t0) continue;
                     const DevTrans &tr = A.tr[t];
-                    const double *f = spec + ((size_t)j * RH_SPEC_ACT + s2i) * RH_SPEC_F;
+                    const float *f = cf[s2i];
                     const float nl = pop[tr.l * N + k], nuu = pop[tr.u * N + k];
                     if (tr.kind == 0) {
                         const float a = __expf((1.0f - sk) * (float)tr.ln_atop + sk * (float)tr.ln_abot);
-                        const float v = ((float)f[3] - vz) * ivth;
-                        const float ph = voigt_f32(a, v, vtab) * (float)(f[4] * kStokesNref) * ivth;
-                        const float Vlu = (float)f[0] * ph;
-                        chi += nl * Vlu - nuu * ((float)f[2] * Vlu);
-                        eta += nuu * ((float)f[1] * ph);
+                        const float v = (f[3] - vz) * ivth;
+                        const float ph = voigt_f32(a, v, vtab) * f[4] * ivth;
+                        const float Vlu = f[0] * ph;
+                        chi += nl * Vlu - nuu * (f[2] * Vlu);
+                        eta += nuu * (f[1] * ph);
                     } else {
                         const float G = gc[tr.sub * N + k] * ex;
-                        const float al = (float)(f[0] * kStokesNref);
-                        chi += nl * al - nuu * G * al;
-                        eta += nuu * G * (float)(f[1] * kStokesNref);
+                        chi += nl * f[0] - nuu * G * f[0];
+                        eta += nuu * G * f[1];
                     }
                 }
                 const float v = (q0 - vz) * ivth;
                 float Hz[3], Lz[3];
-                zeeman_profiles<float>(sf[SF_A0 * N + k], v, sf[SF_VB * N + k], vtab, dtab, Hz, Lz);
+                zeeman_profiles<float>(sf[SF_A0 * N + k], v, sf[SF_VB * N + k], vtab, dtab, nullptr, Hz, Lz);
                 const float s2 = sf[SF_S2 * N + k], ct = sf[SF_CT * N + k];
                 const float c2 = sf[SF_C2 * N + k], sn2 = sf[SF_SN2 * N + k];
                 const float hk = 0.5f * sf[SF_KL * N + k] * hr, Sl = sf[SF_SL * N + k];
@@ -718,7 +705,7 @@ __global__ void __launch_bounds__(128) stokes32_kernel(const __grid_constant__ D
                 const float rq = hk * (Lz[1] - 0.5f * (Lz[0] + Lz[2])) * s2;
                 const float rV = hk * (Lz[2] - Lz[0]) * ct;
                 const float eI = chi + lI;
-                const float ie = 1.0f / eI;
+                const float ie = rcp_f32(eI);
                 const float e6[6] = {lq * c2, lq * sn2, lV, rq * c2, rq * sn2, rV};
                 float Ko[6], So[4];
 #pragma unroll
@@ -876,8 +863,8 @@ cudaError_t launch_start(const DevAtom &A, const ColumnArrays &c, int kind, cons
 
 cudaError_t launch_stokes(const DevAtom &A, const ColumnArrays &c, int t0, double geff, const double *B_T,
                           const double *theta, const double *chi, int64_t nlam, const double *nu_d, const int *nact_d,
-                          const int *act_d, const double *spec_d, const float4 *vtab, const float4 *dtab, double *out,
-                          int precision, cudaStream_t st)
+                          const int *act_d, const double *spec_d, const float4 *vtab, const float4 *dtab,
+                          const double *tab64, double *out, int precision, cudaStream_t st)
 {
     int64_t n = c.ncol * nlam;
     if (n == 0) return cudaSuccess;
@@ -893,18 +880,21 @@ cudaError_t launch_stokes(const DevAtom &A, const ColumnArrays &c, int t0, doubl
         int dev = 0, nsm = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, stokes32_kernel, 128, sm32);
+        // a block walks its wavelengths in equal rounds of at most kStokesThreads
+        const int64_t rounds = (nlam + kStokesThreads - 1) / kStokesThreads;
+        const int th = (int)(((nlam + rounds - 1) / rounds + 31) / 32 * 32);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, stokes32_kernel, th, sm32);
         if (e != cudaSuccess) return e;
         int64_t g = (int64_t)(per > 0 ? per : 1) * nsm;
         if (g > c.ncol) g = c.ncol;
-        stokes32_kernel<<<(unsigned)g, 128, sm32, st>>>(A, c, t0, geff, B_T, theta, chi, nlam, nu_d, nact_d, act_d,
+        stokes32_kernel<<<(unsigned)g, th, sm32, st>>>(A, c, t0, geff, B_T, theta, chi, nlam, nu_d, nact_d, act_d,
                                                         spec_d, vtab, dtab, out);
     } else if (precision == 1)
         stokes_kernel<float><<<(unsigned)blocks, threads, 0, st>>>(A, c, t0, geff, B_T, theta, chi, nlam, nu_d, nact_d,
-                                                                 act_d, spec_d, vtab, dtab, out);
+                                                                 act_d, spec_d, vtab, dtab, tab64, out);
     else
         stokes_kernel<double><<<(unsigned)blocks, threads, 0, st>>>(A, c, t0, geff, B_T, theta, chi, nlam, nu_d,
-                                                                  nact_d, act_d, spec_d, vtab, dtab, out);
+                                                                  nact_d, act_d, spec_d, vtab, dtab, tab64, out);
     return cudaGetLastError();
 }
 

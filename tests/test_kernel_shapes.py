@@ -51,3 +51,24 @@ def test_training_gradients_at_odd_sizes(rh, nbound, ndep, hidden, rows):
             off += size
             assert np.linalg.norm(a - b) < 2e-2 * np.linalg.norm(b) + 1e-12
             assert a @ b > 0.999 * np.linalg.norm(a) * np.linalg.norm(b) - 1e-24
+
+
+@pytest.mark.parametrize("nlam", [1, 31, 224, 225, 401])
+def test_stokes_wavelength_counts(rh, orc, nlam):
+    atom = rh_synth.hydrogen_like_atom()
+    cols = rh_synth.chromosphere_cube(nx=3, ny=1, ndep=21, seed=6)
+    g = rh.Context(0)
+    g.setup_atom(atom)
+    g.load_columns(cols)
+    o = orc.Oracle()
+    o.setup_atom(atom)
+    o.load_columns(cols)
+    n = o.lte()[0] * np.exp(np.random.default_rng(2).uniform(-0.5, 0.5, (3, atom["nlev"], 21)))
+    g.set_populations(n)
+    o.set_populations(n)
+    fld = (np.full((3, 21), 0.15), np.full((3, 21), 0.9), np.full((3, 21), 2.1))
+    lam = 656.46e-9 + np.linspace(-0.4e-9, 0.4e-9, nlam)
+    ref = o.emergent_stokes(4, 1.5, *fld, lam)
+    for prec, tol in ((0, 1e-9), (1, 1e-4)):
+        got = g.emergent_stokes(4, 1.5, *fld, lam, precision=prec)
+        assert np.max(np.abs(got - ref) / ref[..., :1]) < tol
