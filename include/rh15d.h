@@ -411,11 +411,12 @@ int rh_surrogate_file_info(const char *path, int32_t *sizes_out, int64_t *nparam
 /* damping, populations in the working precision, Voigt table, block         */
 /* counters, the warps' line-profile rings) and the carve's end in           */
 /* offsets_out[0..15], and the bytes the launch allocates in bytes_out (the  */
-/* same function sizes and carves, so the two are equal).  macc: rate        */
-/* accumulators per depth.  ring_warps (0..32): warps whose profile ring the */
-/* block holds -- the block's warps for the FP32 kernel with the profile     */
-/* cache and without PRD lines (2304 bytes each: three depths of up to three */
-/* line profiles for the two rays of a sweep pass), 0 for the other kernels. */
+/* same function sizes and carves, so the two are equal).  macc: rows of the  */
+/* rate accumulators per depth (twice the tiles' accumulators where a tile's */
+/* two directions are separate work items).  ring_warps (0..32): units of     */
+/* 2304 bytes of per-warp scratch (profile ring, ray states) that do not fit  */
+/* into the Voigt table's place, which the sweep reuses.  A launch lays out    */
+/* with no collisional-rate region (they are read from device memory).       */
 /* RH_EINVAL for sizes outside the library's limits.                        */
 int rh_column_smem_layout(int32_t precision, int32_t nlev, int32_t ndep, int32_t ntr, int32_t ncont, int32_t nline,
                           int32_t macc, int32_t ring_warps, size_t *offsets_out, size_t *bytes_out);

@@ -379,6 +379,7 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
         da.muf[m] = (float)a.mu[m];
         da.wm2f[m] = (float)(0.5 * a.wmu[m]);
         da.imuf[m] = (float)(1.0 / a.mu[m]);
+        da.imu[m] = 1.0 / a.mu[m];
     }
     for (int t = 0; t < a.ntr; ++t) {
         const HostTrans &h = a.tr[t];
@@ -398,6 +399,7 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
         dt.ln_abot = h.kind == 0 ? std::log(h.a_bot) : 0.0;
     }
     int acc = 0, nmap = 0;
+    std::vector<int> ents[RH_MAXLEV * RH_MAXLEV];   // accumulators of each rate-matrix entry, tile order
     for (int b = 0; b < a.ntile; ++b) {
         const std::vector<int> &un = a.tile_union[b];
         int K = (int)un.size();
@@ -409,10 +411,7 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
         auto add = [&](int accj, int row, int col, int sign) -> bool {
             if (row == col) return true;
             if (nmap >= RH_MAXMAP) return false;
-            da.map_acc[nmap] = (int16_t)(acc + accj);
-            da.map_row[nmap] = (int8_t)row;
-            da.map_col[nmap] = (int8_t)col;
-            da.map_sign[nmap] = (int8_t)sign;
+            ents[row * RH_MAXLEV + col].push_back((acc + accj) * 2 + (sign < 0 ? 1 : 0));
             ++nmap;
             return true;
         };
@@ -435,7 +434,26 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
         acc += tl.m;
     }
     da.macc = acc;
-    da.nmap = nmap;
+    {
+        int o = 0, x = 0, ne = 0;
+        for (int rc = 0; rc < RH_MAXLEV * RH_MAXLEV; ++rc) {
+            std::vector<int> cx;
+            for (int t = 0; t < a.ntr; ++t)
+                for (int down = 0; down < 2; ++down)
+                    if ((down ? a.tr[t].l : a.tr[t].u) * RH_MAXLEV + (down ? a.tr[t].u : a.tr[t].l) == rc)
+                        cx.push_back(2 * t + down);
+            da.ent_id[rc] = -1;
+            if (ents[rc].empty() && cx.empty()) continue;
+            da.ent_id[rc] = (int8_t)ne;
+            da.ent_off[ne] = (int16_t)o;
+            da.cx_off[ne] = (int8_t)x;
+            for (int m : ents[rc]) da.ent_acc[o++] = (int16_t)m;
+            for (int m : cx) da.cx_idx[x++] = (int8_t)m;
+            da.ent_off[++ne] = (int16_t)o;
+            da.cx_off[ne] = (int8_t)x;
+        }
+        da.nent = ne;
+    }
     // profile-cache rows: one per line slot of every tile
     da.nphi = 0;
     for (int b = 0; b < a.ntile; ++b) {
@@ -446,7 +464,9 @@ int build_atom(rh_ctx *c, const rh_atom_desc *d)
                 da.phi_tile[da.nphi] = (int16_t)b;
                 da.phi_j[da.nphi] = (int8_t)j;
                 tl.phi[j] = da.nphi++;
+                tl.nl++;
             }
+        da.maxnl = std::max(da.maxnl, tl.nl);
     }
     // partial redistribution
     {
@@ -653,6 +673,7 @@ void set_phic(const rh_ctx *c, IterLaunch &il)
 {
     il.phic = c->phic;
     il.phic_cap = c->phic_cap;
+    il.tab64 = c->tab64_d;
 }
 
 void set_prd(const rh_ctx *c, IterLaunch &il, double eps0, int hybrid)
@@ -1056,7 +1077,7 @@ int rh_create(rh_ctx **out, int cuda_device, void *cuda_stream)
     }
     if (e == cudaSuccess) e = cudaMalloc(&c->dtab_d, (RH_VT_N + 1) * sizeof(float4));
     if (e == cudaSuccess) e = cudaMemcpy(c->dtab_d, dt.data(), (RH_VT_N + 1) * sizeof(float4), cudaMemcpyHostToDevice);
-    const std::vector<double> t64 = math64_table();
+    const std::vector<double> &t64 = math64_table();
     if (e == cudaSuccess) e = cudaMalloc(&c->tab64_d, t64.size() * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpy(c->tab64_d, t64.data(), t64.size() * sizeof(double), cudaMemcpyHostToDevice);
     *out = c;

@@ -45,25 +45,33 @@ struct DevTile {
     int prd_slot;                 // slot j of a PRD line in the union, -1: none
     int pacc_off;                 // first plain-rate accumulator (2 per slot), PRD atoms only
     int phi[RH_KMAX];             // line slot: its row of the profile cache; -1: continuum
+    int nl;                       // lines of the union (they come first)
 };
 
 // Everything the column kernel needs about the atom, passed by value as a
 // __grid_constant__ kernel parameter (read through the constant bank).
 struct DevAtom {
-    int nlev, ntr, nline, ncont, ntile, nmu, macc, nmap;
+    int nlev, ntr, nline, ncont, ntile, nmu, macc;
     double mass, metal_floor;
     double lev_chi[RH_MAXLEV];    // E_continuum - E_i, J (bound levels)
     double lev_g2[RH_MAXLEV];     // g_i / (2 g_continuum)
     double mu[RH_MAXMU], wmu[RH_MAXMU];
     float muf[RH_MAXMU], wm2f[RH_MAXMU];   // mu and w_mu / 2 for the FP32 sweep
     float imuf[RH_MAXMU];                    // 1/mu
+    double imu[RH_MAXMU];
+    int maxnl;                               // most line slots of any tile
     DevTrans tr[RH_MAXTR];
     double col_c[RH_MAXTR];       // collisional rates: line f / dE, continuum alpha0 / (h nu0)
     DevTile tile[RH_MAXTILE];
     int16_t order[RH_MAXTILE];               // tile processing order (most expensive first)
-    // accumulator -> rate-matrix entry map: A[row][col] += sign * acc
-    int16_t map_acc[RH_MAXMAP];
-    int8_t map_row[RH_MAXMAP], map_col[RH_MAXMAP], map_sign[RH_MAXMAP];
+    // off-diagonal rate-matrix entries in use, e = 0 .. nent - 1 (ent_id[row *
+    // RH_MAXLEV + col], -1: zero): the sum over i in ent_off[e] .. ent_off[e + 1]
+    // of the accumulators ent_acc[i] >> 1 (bit 0: subtracted) plus the
+    // collisional rates cx_idx[cx_off[e] .. cx_off[e + 1]] of the column's list
+    int nent;
+    int8_t ent_id[RH_MAXLEV * RH_MAXLEV];
+    int16_t ent_off[RH_MAXLEV * RH_MAXLEV + 1], ent_acc[RH_MAXMAP];
+    int8_t cx_off[RH_MAXLEV * RH_MAXLEV + 1], cx_idx[2 * RH_MAXTR];
     // partial redistribution: PRD lines, their points (offsets into the point
     // arrays, frequency order) and redistribution-kernel blocks (offsets, np^2)
     int nprd, npp, pacc;
@@ -748,6 +756,7 @@ struct IterLaunch {
     // evaluates the Voigt profiles itself
     void *phic = nullptr;
     size_t phic_cap = 0;
+    const double *tab64 = nullptr;            // FP64 function tables (rh15d_math64.h)
 };
 cudaError_t launch_mali(const DevAtom &A, const ColumnArrays &c, const void *lane_tab, int npad,
                         const float4 *vtab, double nref, double *nghist, size_t nghist_cap, int *queue,

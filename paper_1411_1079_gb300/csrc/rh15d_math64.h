@@ -11,11 +11,12 @@
 //     Dawson's integral, w(z) = e^{-z^2} + (2i/sqrt pi) F(z), so that
 //       H = e^{a^2 - v^2} cos 2av - (2/sqrt pi) [a F' - a^3/6 F''' + a^5/120 F^(5) - ...],
 //       L = -e^{a^2 - v^2} sin 2av + (2/sqrt pi) [F - a^2/2 F'' + a^4/24 F^(4) - ...],
-//     F and F' for |v| < 8 from their Taylor polynomials (degree 11) about
-//     the centres of 64 intervals (both tabulated: F' = 1 - 2vF cancels),
+//     F and F' for |v| < 16 from their Taylor polynomials (degree 11) about
+//     the centres of 128 intervals (both tabulated: F' = 1 - 2vF cancels),
 //     the higher derivatives from F^(n+1) = -2 (v F^(n) + n F^(n-1)); for
-//     |v| >= 8 the asymptotic series of w with as many terms as |v| needs
-//     (8 to 17).  About 85 FP64 operations against some thousands of the
+//     |v| >= 16 the asymptotic series of w with as many terms as |v| needs
+//     (6 to 10; the lanes of a warp reach from a line's core into its wings
+//     and run both branches, so the branch point is where the second is short).  About 85 FP64 operations against some thousands of the
 //     Dawson power series (voigt_f64, used for the host's tables), error
 //     below 2e-15 relative where the series has up to 1e-14 (F' cancels
 //     there).
@@ -27,16 +28,17 @@
 
 namespace rh {
 
-constexpr int kV64N = 64;            // intervals of the Dawson tables
-constexpr double kV64Max = 8.0;      // their range in |v|
+constexpr int kV64N = 128;           // intervals of the Dawson tables
+constexpr double kV64Max = 16.0;     // their range in |v|
 constexpr int kV64Deg = 12;          // coefficients per polynomial
 constexpr int kV64Row = 25;          // doubles per interval: F then F' (odd: spreads shared-memory banks)
 constexpr int kT64Exp = kV64N * kV64Row;        // offset of 2^{j/64}
 constexpr int kT64Dfac = kT64Exp + 64;          // offset of (2k-1)!!
 constexpr int kT64Size = kT64Dfac + 18;         // doubles of the whole table
 
-// The table, in long double on the host (rounded once).
-inline std::vector<double> math64_table()
+// The table, in long double on the host (rounded once; computed once per
+// process: long double is emulated on some hosts, 3 ms).
+inline std::vector<double> math64_table_build()
 {
     std::vector<double> t(kT64Size, 0.0);
     for (int j = 0; j < kV64N; ++j) {
@@ -51,9 +53,7 @@ inline std::vector<double> math64_table()
         }
         long double a[kV64Deg + 2];
         a[0] = expl(-c * c) * s;
-        // the series loses nothing (positive terms); a_1 = F' through its
-        // asymptotic form where 1 - 2cF cancels
-        a[1] = 1.0L - 2.0L * c * a[0];
+        a[1] = 1.0L - 2.0L * c * a[0];   // F', through its asymptotic form where this cancels
         if (c > 5.0L) {
             long double u = 1.0L / (2.0L * c * c), p = 1.0L, sum = 0.0L, last = 1e30L;
             for (int k = 1; k < 60; ++k) {
@@ -77,6 +77,12 @@ inline std::vector<double> math64_table()
         t[kT64Dfac + k] = f;   // (2k-1)!!
         f *= 2 * k + 1;
     }
+    return t;
+}
+
+inline const std::vector<double> &math64_table()
+{
+    static const std::vector<double> t = math64_table_build();
     return t;
 }
 
@@ -179,7 +185,7 @@ __device__ __forceinline__ void voigt64(double a, double v, const double *__rest
         o = fma(o, a2, D[5] * (1.0 / 120));
         o = fma(o, a2, D[3] * (-1.0 / 6));
         o = fma(o, a2, D[1]);
-        const double th2 = 4.0 * a2 * av * av;   // (2av)^2 <= 0.64
+        const double th2 = 4.0 * a2 * av * av;   // (2av)^2 <= 0.4 where e^{-v^2} counts
         // e^{a^2 - v^2}; a^2 <= 0.0025
         const double g = exp64(fma(a, a, -av * av), tab);
         double cs = fma(th2, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
@@ -210,7 +216,8 @@ __device__ __forceinline__ void voigt64(double a, double v, const double *__rest
     }
     // w = (i / (sqrt(pi) z)) sum_k (2k-1)!! u^k, u = 1/(2z^2); the k-th term
     // over the first is below 1e-17 from k = K on
-    const int K = av < 10.0 ? 17 : (av < 14.0 ? 13 : (av < 24.0 ? 10 : 8));
+    // (e^{-v^2} < 2e-111 here)
+    const int K = av < 24.0 ? 10 : (av < 60.0 ? 8 : 6);
     const double v2 = av * av, a2 = a * a;
     const double zr = 2.0 * (v2 - a2), zi = 4.0 * av * a;
     const double id = rcp64(fma(zr, zr, zi * zi));
@@ -225,11 +232,6 @@ __device__ __forceinline__ void voigt64(double a, double v, const double *__rest
     const double im = rcp64(1.77245385090551602730 * (v2 + a2));
     H = (sr * a - si * av) * im;
     if (DISP) L = (sr * av + si * a) * im;
-    if (v2 < 110.0) {   // e^{-v^2} < 2e-48 beyond
-        const double g = exp64(a2 - v2, tab);
-        H += g * cos(2.0 * av * a);
-        if (DISP) L -= g * sin(2.0 * av * a);
-    }
     if (DISP) L = v < 0.0 ? -L : L;
 }
 #endif

@@ -53,6 +53,25 @@ def test_training_gradients_at_odd_sizes(rh, nbound, ndep, hidden, rows):
             assert a @ b > 0.999 * np.linalg.norm(a) * np.linalg.norm(b) - 1e-24
 
 
+@pytest.mark.parametrize("nmu", [1, 2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("nbound,ndep", [(2, 2), (3, 33), (6, 12)])
+def test_column_kernel_over_angles_and_levels(rh, orc, nmu, nbound, ndep):
+    atom = rh_synth.small_atom(nbound=nbound, nmu=nmu)
+    cols = rh_synth.chromosphere_cube(nx=5, ny=1, ndep=ndep, seed=3)
+    g = rh.Context(0)
+    g.setup_atom(atom)
+    o = orc.Oracle()
+    o.setup_atom(atom)
+    for formal in (0, 1):
+        g.load_columns(cols)
+        o.load_columns(cols)
+        o.iterate(maxiter=4, tol=0.0, ng_order=0, formal=formal)
+        no = o.populations()[0]
+        for prec, tol in ((0, 1e-9), (1, 1e-3)):
+            g.iterate(maxiter=4, tol=0.0, ng_order=0, precision=prec, formal=formal)
+            assert np.max(np.abs(g.populations()[0] / no - 1)) < tol, (formal, prec)
+
+
 @pytest.mark.parametrize("nlam", [1, 31, 224, 225, 401])
 def test_stokes_wavelength_counts(rh, orc, nlam):
     atom = rh_synth.hydrogen_like_atom()
