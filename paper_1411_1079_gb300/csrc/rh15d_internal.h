@@ -107,13 +107,9 @@ constexpr int kLaneFields = kLaneNu + 4;
 constexpr double kNuRef3 = 1e45;   // (1e15 Hz)^3: free-free coefficient scale
 
 // ----------------------------------------------------------------------------
-// Voigt function H(a, v), FP64 (FP64 path and table set-up).
-// |v| < 6: Taylor expansion of w(v + i a) in the damping a about the real
-// axis, w(v) = exp(-v^2) + (2i/sqrt(pi)) F(v) with Dawson's integral F from
-// its positive power series F(v) = exp(-v^2) sum v^{2n+1} / (n! (2n+1)), and
-// the derivatives from w' = -2 z w + 2i/sqrt(pi), w^{(n+1)} = -2 z w^{(n)} -
-// 2 n w^{(n-1)} (order 9; a <= 0.05).  |v| >= 6: w(z) ~ exp(-z^2) +
-// (i / (sqrt(pi) z)) sum_k (2k-1)!! / (2 z^2)^k, 36 terms.  ~1e-13 relative.
+// Dawson's integral from its positive power series F(v) = exp(-v^2) sum
+// v^{2n+1} / (n! (2n+1)) (set-up of the FP32 tables; the FP64 Voigt function is
+// in rh15d_math64.h).
 __host__ __device__ inline double dawson_series(double x)
 {
     double s = 0.0, term = x, x2 = x * x;
@@ -124,105 +120,6 @@ __host__ __device__ inline double dawson_series(double x)
         term *= x2 / (n + 1);
     }
     return exp(-x2) * s;
-}
-
-__host__ __device__ inline double voigt_f64(double a, double v)
-{
-    double av = fabs(v);
-    if (av < 6.0) {
-        // w and derivatives at the real point v (complex as re/im pairs)
-        double e = exp(-av * av);
-        double F = dawson_series(av);
-        double wr[10], wi[10];
-        wr[0] = e;
-        wi[0] = 2.0 / kSqrtPi * F;
-        wr[1] = -2.0 * av * wr[0];
-        wi[1] = -2.0 * av * wi[0] + 2.0 / kSqrtPi;
-        for (int n = 1; n < 9; ++n) {
-            wr[n + 1] = -2.0 * (av * wr[n] + n * wr[n - 1]);
-            wi[n + 1] = -2.0 * (av * wi[n] + n * wi[n - 1]);
-        }
-        // sum_n (i a)^n / n! w^{(n)}: real part
-        double h = 0.0, pw = 1.0;
-        for (int n = 0; n <= 9; ++n) {
-            switch (n & 3) {
-            case 0: h += pw * wr[n]; break;
-            case 1: h -= pw * wi[n]; break;
-            case 2: h -= pw * wr[n]; break;
-            default: h += pw * wi[n]; break;
-            }
-            pw *= a / (n + 1);
-        }
-        return h;
-    }
-    // asymptotic: z = av + i a; w = exp(-z^2) + (i/(sqrt(pi) z)) S,
-    // S = sum t_k, t_{k+1} = t_k (2k+1)/(2 z^2)
-    double zr = av, zi = a;
-    double z2r = 2.0 * (zr * zr - zi * zi), z2i = 2.0 * (2.0 * zr * zi);
-    double d = z2r * z2r + z2i * z2i;
-    double ir = z2r / d, ii = -z2i / d;   // 1/(2 z^2)
-    double sr = 0.0, si = 0.0, tr = 1.0, ti = 0.0;
-    for (int k = 0; k <= 36; ++k) {
-        sr += tr;
-        si += ti;
-        double nr = (tr * ir - ti * ii) * (2 * k + 1), ni = (tr * ii + ti * ir) * (2 * k + 1);
-        tr = nr;
-        ti = ni;
-    }
-    // Re[i S conj(z)] / (sqrt(pi)|z|^2) with i S = (-si) + i sr
-    double mz = zr * zr + zi * zi;
-    return (-si * zr + sr * zi) / (kSqrtPi * mz) + exp(zi * zi - zr * zr) * cos(2.0 * zr * zi);
-}
-
-// Faddeeva function w(v + i a) = H + i L, FP64, by the same two branches as
-// voigt_f64 (Taylor expansion in a about the real axis for |v| < 6, the
-// asymptotic series above); H is even and L odd in v.
-__host__ __device__ inline void faddeeva_f64(double a, double v, double &H, double &L)
-{
-    double av = fabs(v), sg = v < 0.0 ? -1.0 : 1.0;
-    if (av < 6.0) {
-        double e = exp(-av * av);
-        double F = dawson_series(av);
-        double wr[10], wi[10];
-        wr[0] = e;
-        wi[0] = 2.0 / kSqrtPi * F;
-        wr[1] = -2.0 * av * wr[0];
-        wi[1] = -2.0 * av * wi[0] + 2.0 / kSqrtPi;
-        for (int n = 1; n < 9; ++n) {
-            wr[n + 1] = -2.0 * (av * wr[n] + n * wr[n - 1]);
-            wi[n + 1] = -2.0 * (av * wi[n] + n * wi[n - 1]);
-        }
-        // sum_n (i a)^n / n! w^{(n)}: real and imaginary parts
-        double h = 0.0, l = 0.0, pw = 1.0;
-        for (int n = 0; n <= 9; ++n) {
-            switch (n & 3) {
-            case 0: h += pw * wr[n]; l += pw * wi[n]; break;
-            case 1: h -= pw * wi[n]; l += pw * wr[n]; break;
-            case 2: h -= pw * wr[n]; l -= pw * wi[n]; break;
-            default: h += pw * wi[n]; l -= pw * wr[n]; break;
-            }
-            pw *= a / (n + 1);
-        }
-        H = h;
-        L = sg * l;
-        return;
-    }
-    double zr = av, zi = a;
-    double z2r = 2.0 * (zr * zr - zi * zi), z2i = 2.0 * (2.0 * zr * zi);
-    double d = z2r * z2r + z2i * z2i;
-    double ir = z2r / d, ii = -z2i / d;
-    double sr = 0.0, si = 0.0, tr = 1.0, ti = 0.0;
-    for (int k = 0; k <= 36; ++k) {
-        sr += tr;
-        si += ti;
-        double nr = (tr * ir - ti * ii) * (2 * k + 1), ni = (tr * ii + ti * ir) * (2 * k + 1);
-        tr = nr;
-        ti = ni;
-    }
-    // w = i S conj(z) / (sqrt(pi)|z|^2) + exp(-z^2)
-    double mz = zr * zr + zi * zi, ez = exp(zi * zi - zr * zr);
-    H = (-si * zr + sr * zi) / (kSqrtPi * mz) + ez * cos(2.0 * zr * zi);
-    L = sg * ((sr * zr + si * zi) / (kSqrtPi * mz) - ez * sin(2.0 * zr * zi));
 }
 
 // Coefficients of the expansion of the dispersion function in the damping a

@@ -17,7 +17,7 @@
 //     |v| >= 16 the asymptotic series of w with as many terms as |v| needs
 //     (6 to 10; the lanes of a warp reach from a line's core into its wings
 //     and run both branches, so the branch point is where the second is short).  About 85 FP64 operations against some thousands of the
-//     Dawson power series (voigt_f64, used for the host's tables), error
+//     Dawson power series (one division a term, up to 130 terms), error
 //     below 2e-15 relative where the series has up to 1e-14 (F' cancels
 //     there).
 #pragma once
