@@ -1225,7 +1225,7 @@ int rh_load_columns(rh_ctx *c, int64_t ncol, int32_t ndep, const double *z_m, co
     }
     c->ncol = ncol;
     c->ndep = ndep;
-    CK(launch_lte_setup(c->da, a, ne_m3 ? 1 : 0, c->st));
+    CK(launch_lte_setup(c->da, a, ne_m3 ? 1 : 0, c->tab64_d, c->st));
     CK(cudaStreamSynchronize(c->st));
     // reference density of the FP32 population scaling: a fixed constant, so
     // that a column's result does not depend on which other columns are

@@ -572,36 +572,18 @@ __device__ __forceinline__ void sc_weights(R d, R &one_m_e0, R &wu, R &wo)
     sc_weights(d, one_m_e0, wu, wo, omwo);
 }
 
-// e^y E1(y), y > 0: series (y <= 1) or the continued fraction
-// E1(y) = e^{-y} / (y + 1 - 1^2/(y + 3 - 2^2/(y + 5 - ...))) evaluated with
-// the modified Lentz algorithm.
-__host__ __device__ inline double exp_e1(double y)
+// e^y E1(y) for 0 < y <= 1: E1 = -gamma - ln y - sum (-y)^n / (n n!), 18 terms
+// (the next is below 1e-18)
+__device__ __forceinline__ double exp_e1_small(double y)
 {
-    if (y <= 1.0) {
-        const double gam = 0.57721566490153286061;
-        double s = 0.0, t = 1.0;
-        for (int n = 1; n < 100; ++n) {
-            t *= -y / n;
-            double a = t / n;
-            s += a;
-            if (fabs(a) < 1e-18 * fabs(s) + 1e-300) break;
-        }
-        return exp(y) * (-gam - log(y) - s);
+    const double gam = 0.57721566490153286061;
+    double s = 0.0, t = 1.0;
+#pragma unroll
+    for (int n = 1; n <= 18; ++n) {
+        t *= -y * (1.0 / n);
+        s = fma(t, 1.0 / n, s);
     }
-    const double tiny = 1e-300;
-    double f = y + 1.0, C = f, D = 0.0;
-    for (int n = 1; n < 500; ++n) {
-        double an = -(double)n * n, bn = y + 2.0 * n + 1.0;
-        D = bn + an * D;
-        if (fabs(D) < tiny) D = tiny;
-        C = bn + an / C;
-        if (fabs(C) < tiny) C = tiny;
-        D = 1.0 / D;
-        double delta = C * D;
-        f *= delta;
-        if (fabs(delta - 1.0) < 1e-16) break;
-    }
-    return 1.0 / f;
+    return exp(y) * (-gam - log(y) - s);
 }
 
 // H- bound-free cross section (John 1988 fit), m^2; lambda in m.
@@ -624,7 +606,7 @@ struct ColumnArrays {
 };
 
 // launchers (defined in the kernel translation units)
-cudaError_t launch_lte_setup(const DevAtom &A, const ColumnArrays &c, int ne_given, cudaStream_t st);
+cudaError_t launch_lte_setup(const DevAtom &A, const ColumnArrays &c, int ne_given, const double *tab64, cudaStream_t st);
 struct IterLaunch {
     int precision = 1, persistent = 1, block_warps = 0, maxiter = 1, ng_order = 0, ng_delay = 0, ng_period = 1,
         start = 0;

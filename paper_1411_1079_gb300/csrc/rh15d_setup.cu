@@ -21,8 +21,11 @@ namespace {
 // few: one exponential per level, from which every transition's Boltzmann
 // factor e^{-y} follows as a ratio, one reciprocal per level, and E1 only
 // where it decides P (y < 1: the closest pairs of levels).
-// 65536 x 82 points, 15 transitions: rh_load_columns 101.7 -> 13.3 ms.
-__global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, int ne_given)
+// 65536 x 82 points, 15 transitions: rh_load_columns 101.7 -> 13.3 ms,
+// with the table-driven exponential, Newton reciprocals and E1's series without
+// divisions (and the kept arrays) 6.3 ms.
+__global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, int ne_given,
+                                 const double *__restrict__ tab64)
 {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int N = c.ndep, L = A.nlev;
@@ -37,7 +40,8 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
     double phi[RH_MAXLEV], ex[RH_MAXLEV];   // ex: exp((E_continuum - E_i) / kT)
     double Phi = 0.0;
     for (int i = 0; i < ic; ++i) {
-        ex[i] = exp(div64(A.lev_chi[i], kT, ikT));
+        const double x = div64(A.lev_chi[i], kT, ikT);
+        ex[i] = x < 700.0 ? exp64(x, tab64) : exp(x);
         phi[i] = A.lev_g2[i] * lam3 * ex[i];
         Phi += phi[i];
     }
@@ -57,8 +61,8 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
     ns[ic] = nc;
     c.np[idx] = nc;
     for (int i = 0; i < L; ++i) {
-        ins[i] = 1.0 / ns[i];
-        iex[i] = 1.0 / ex[i];
+        ins[i] = rcp64(ns[i]);
+        iex[i] = rcp64(ex[i]);
         c.nstar[((size_t)col * L + i) * N + k] = ns[i];
         c.pops[((size_t)col * L + i) * N + k] = ns[i];
     }
@@ -73,7 +77,7 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
         if (tr.kind == 0) {
             // g_l cancels with 1/g_l; e^y E1(y) falls with y and is 0.5963 at
             // y = 1, below 0.2/0.276: P is 0.2 from there on
-            const double P = y >= 1.0 ? 0.2 : fmax(0.2, 0.276 * exp_e1(y));
+            const double P = y >= 1.0 ? 0.2 : fmax(0.2, 0.276 * exp_e1_small(y));
             up = neK * A.col_c[t] * P * ey;
         } else {
             up = neS * A.col_c[t] * ey * kT;
@@ -839,13 +843,13 @@ __global__ void regrid_kernel(int64_t ncol, int N, int M, const double *z, const
 
 }  // namespace
 
-cudaError_t launch_lte_setup(const DevAtom &A, const ColumnArrays &c, int ne_given, cudaStream_t st)
+cudaError_t launch_lte_setup(const DevAtom &A, const ColumnArrays &c, int ne_given, const double *tab64, cudaStream_t st)
 {
     int64_t n = c.ncol * c.ndep;
     if (n == 0) return cudaSuccess;
     int threads = 128;
     int64_t blocks = (n + threads - 1) / threads;
-    lte_setup_kernel<<<(unsigned)blocks, threads, 0, st>>>(A, c, ne_given);
+    lte_setup_kernel<<<(unsigned)blocks, threads, 0, st>>>(A, c, ne_given, tab64);
     return cudaGetLastError();
 }
 
