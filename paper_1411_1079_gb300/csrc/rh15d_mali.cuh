@@ -612,8 +612,8 @@ __device__ __forceinline__ void planck_terms(double x, const double *tab, double
 }
 
 // Element of the profile cache for cache row `row`, direction dir, depth k,
-// angle m and lane: [row][dir][depth] blocks of nmu x 32 values, in FP32 two
-// angles interleaved (the vectors of the sweep), the last of an odd number of
+// angle m and lane: [row][dir][depth] blocks of nmu x 32 values; PAIRS (the FP32
+// kernels of sweep_unit): two angles interleaved, the last of an odd number of
 // angles alone.  (int: at most 288 rows x 2 x 4096 depths x 8 angles x 32
 // lanes < 2^31)
 template <typename R>
@@ -621,11 +621,18 @@ __device__ __forceinline__ int phi_block(int nmu, int N, int row, int dir, int k
 {
     return ((row * 2 + dir) * N + k) * (nmu * kWarp);
 }
-template <typename R>
+template <bool PAIRS>
 __device__ __forceinline__ int phi_elem(int nmu, int m, int lane)
 {
-    if (sizeof(R) == 8 || ((nmu & 1) && m == nmu - 1)) return m * kWarp + lane;
+    if (!PAIRS || ((nmu & 1) && m == nmu - 1)) return m * kWarp + lane;
     return (m >> 1) * 2 * kWarp + 2 * lane + (m & 1);
+}
+
+// The kernels of sweep_tile_k walk one ray at a time and keep a ray's depths
+// together: [row][dir][angle][depth][32 lanes]; first element of a ray.
+__device__ __forceinline__ int phi_ray(int nmu, int N, int row, int dir, int m)
+{
+    return ((row * 2 + dir) * nmu + m) * N * kWarp;
 }
 
 // Depth-dependent, angle-independent quantities of one lane (NL lines first,
@@ -775,7 +782,7 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p,
                 const int m1 = 2 * (v0 + v), m2 = m1 + 1 < nmu ? m1 + 1 : m1;
                 if constexpr (CACHE) {
                     const R *c = phc + poff[j] + k * blk;
-                    return pk(c[phi_elem<R>(nmu, m1, lane)], c[phi_elem<R>(nmu, m2, lane)]);
+                    return pk(c[phi_elem<sizeof(R) == 4>(nmu, m1, lane)], c[phi_elem<sizeof(R) == 4>(nmu, m2, lane)]);
                 } else {
                     const R a = s.ad[lc.sub[j] * N + k], z1 = dir ? A.muf[m1] : -A.muf[m1],
                             z2 = dir ? A.muf[m2] : -A.muf[m2];
@@ -784,7 +791,7 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p,
                 }
             } else {
                 const int m = v0 + v;
-                if constexpr (CACHE) return phc[poff[j] + k * blk + phi_elem<R>(nmu, m, lane)];
+                if constexpr (CACHE) return phc[poff[j] + k * blk + phi_elem<sizeof(R) == 4>(nmu, m, lane)];
                 else
                     return line_phi(lc.q[j], dir ? A.mu[m] : -A.mu[m], s.vz[k], s.ivth[k], s.ad[lc.sub[j] * N + k],
                                     lc.pn[j], s.vtab, tab);
@@ -1073,14 +1080,14 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
     // line profiles of depth k, ray r (2 m + d) for the tile's line slots (0
     // elsewhere): read from the column's cache (CACHE), or evaluated here (the
     // same arithmetic as the cache's build)
+    int pb[K];                                     // the ray's first element of each line slot's cache rows
     auto load_ph = [&](int k, int r, R (&o)[K]) {
-        const int el = phi_elem<R>(nmu, r >> 1, lane);
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             if (!lc.isline[j]) {
                 o[j] = 0;
             } else if constexpr (CACHE) {
-                o[j] = phc[phi_block<R>(nmu, N, tl.phi[j], r & 1, k) + el];
+                o[j] = phc[pb[j] + k * kWarp];
             } else {
                 const R mu = mu_of<R>(A, r >> 1);
                 o[j] = line_phi(lc.q[j], (r & 1) ? mu : -mu, s.vz[k], s.ivth[k], s.ad[lc.sub[j] * N + k], lc.pn[j],
@@ -1175,6 +1182,9 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
         for (int dir = dir0; dir < dir1; ++dir) {
             const R muz = dir == 0 ? -mu : mu;
             const int ray = 2 * m + dir;
+#pragma unroll
+            for (int j = 0; j < K; ++j)
+                pb[j] = CACHE && lc.isline[j] ? phi_ray(nmu, N, tl.phi[j], dir, m) + lane : 0;
             R I, chip = 0, Sp;
             // rho of the lane's PRD point: the static-frame ratio, or (hybrid)
             // this ray's interpolated gas-frame ratio
@@ -1284,9 +1294,11 @@ __device__ __forceinline__ void sweep_tile(const DevAtom &A, const Smem<R> &s, c
     R *slot = s.slot + (size_t)(tl.acc_off + (p.split && d0 ? A.macc : 0)) * p.N;
 #define RH_TILE(K_, NL_) \
     sweep_tile_k<R, K_, NL_, PRD, CACHE, BEZ>(A, s, p, b, d0, d1, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc)
-    if constexpr (sizeof(R) == 4) {
+    if constexpr (sizeof(R) == 4 && !PRD) {
         // the slots' kinds at compile time (Bezier, 300 columns x 8 iterations:
-        // 25.8 -> 23.5 ms; FP64 is bound by its arithmetic and keeps them at run time)
+        // 25.8 -> 23.5 ms; with partial redistribution the nine tile bodies cost
+        // more in instruction fetches than they save, 3.2 -> 4.8 ms an iteration of
+        // 304 columns, and FP64 is bound by its arithmetic)
         switch (tl.K * 4 + tl.nl) {
         case 4: RH_TILE(1, 0); break;
         case 5: RH_TILE(1, 1); break;
@@ -1439,7 +1451,7 @@ __device__ void hybrid_JD(const DevAtom &A, const PrdScr<R> &ps, int N)
 
 // Fill the column's profile cache: warps take (row, direction, quarter of the
 // depths), lanes their wavelengths (the same arithmetic as the uncached sweep).
-template <typename R>
+template <typename R, bool UNITS, bool PAIRS>
 __device__ void build_profiles(const DevAtom &A, const Smem<R> &s, const KParams &p, R *phc)
 {
     const int N = p.N, nmu = A.nmu;
@@ -1460,12 +1472,14 @@ __device__ void build_profiles(const DevAtom &A, const Smem<R> &s, const KParams
                 return line_phi(q, dir ? mu : -mu, vz, iv, a, pn, s.vtab, p.tab64);
             };
             int m = 0;
-            if (sizeof(R) == 4)
+            if (!UNITS)
+                for (; m < nmu; ++m) phc[phi_ray(nmu, N, row, dir, m) + k * kWarp + lane] = at(m);
+            if (PAIRS)
                 for (; m + 1 < nmu; m += 2) {
                     const float2 v = make_float2(at(m), at(m + 1));
-                    *reinterpret_cast<float2 *>(o + phi_elem<R>(nmu, m, lane)) = v;
+                    *reinterpret_cast<float2 *>(o + phi_elem<PAIRS>(nmu, m, lane)) = v;
                 }
-            for (; m < nmu; ++m) o[phi_elem<R>(nmu, m, lane)] = at(m);
+            for (; m < nmu; ++m) o[phi_elem<PAIRS>(nmu, m, lane)] = at(m);
         }
     }
 }
@@ -1649,7 +1663,7 @@ __device__ __forceinline__ int solve_depth(const DevAtom &A, const R *slot, int 
 // redistribution), -1: the kernels of sweep_tile_k.  FP32: 128 registers, two
 // resident blocks of 256 threads or one of 512.
 template <typename R, bool PRD, bool CACHE, bool BEZ, int NV>
-__global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1) mali_kernel(const __grid_constant__ DevAtom A, const __grid_constant__ KParams p)
+__global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(R) == 4 && NV < 0 ? 2 : 1) mali_kernel(const __grid_constant__ DevAtom A, const __grid_constant__ KParams p)
 {
     extern __shared__ __align__(16) char smem_raw[];
     const int N = p.N, L = A.nlev;
@@ -1709,7 +1723,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256, 1) mali_kernel(con
         const double *Cr = p.Crate + cN * 2 * A.ntr;
         if (phc) {
             __syncthreads();   // the column's Doppler widths, velocities and damping
-            build_profiles<R>(A, s, p, phc);
+            build_profiles<R, UNITS, UNITS && sizeof(R) == 4>(A, s, p, phc);
         }
         if constexpr (PRD) {
             // redistribution kernels of the column: K_ij = R(x_j, x_i) w_j / sum_j (.),
