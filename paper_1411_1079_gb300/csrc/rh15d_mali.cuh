@@ -1179,7 +1179,8 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
 
     for (int m = 0; m < nmu; ++m) {
         const R mu = mu_of<R>(A, m), imu = imu_of<R>(A, m), wm2 = wm2_of<R>(A, m);
-        for (int dir = dir0; dir < dir1; ++dir) {
+        // (partial redistribution: always both, a trip count the compiler knows)
+        for (int dir = PRD ? 0 : dir0; dir < (PRD ? 2 : dir1); ++dir) {
             const R muz = dir == 0 ? -mu : mu;
             const int ray = 2 * m + dir;
 #pragma unroll
