@@ -55,7 +55,7 @@ struct Shape {
 // accumulators are the largest part of the shared memory): twice the items
 // balance the warps (20 tiles on 8 warps: 3 rounds of both directions, 5 of
 // one): 1000 columns x 12 iterations 42 -> 20 ms, one column 6.4 -> 5.8 ms,
-// Bezier 300 columns 33 -> 21 ms, FP64 43.0 -> 42.4 ms.
+// FP64 43.0 -> 42.4 ms.
 cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool bez, int bw, Shape &s)
 {
     const bool f32 = precision == 1, units = !A.nprd && !bez;
@@ -68,7 +68,7 @@ cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool be
                       : 3 * A.nmu * kWarp * (int)sizeof(double);
     s.nvp = s.piece ? (int)(kVtabBytes / s.piece) : 0;
     const int extra = s.piece && bw > s.nvp ? ((bw - s.nvp) * s.piece + kScratchUnit - 1) / kScratchUnit : 0;
-    for (int split = 0; split <= (A.nprd ? 0 : 1); ++split) {
+    for (int split = 0; split <= (units ? 1 : 0); ++split) {
         // accumulators (of both directions), or the rate-matrix entries summed in their place
         const int macc = std::max(split ? 2 * A.macc : A.macc, (f32 ? 2 : 1) * A.nent);
         const size_t sm = f32 ? smem_bytes<float>(A.nlev, N, 0, A.ncont, A.nline, macc, extra)

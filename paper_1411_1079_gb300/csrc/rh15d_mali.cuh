@@ -1041,15 +1041,12 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p,
 // and depth from the block's scratch), PRD lanes accumulate the angle-averaged
 // mean intensity J, and every slot also accumulates its plain rates (actual
 // intensity) cw I and cw R (E + I), for the PRD update.
-// NL >= 0: the tile's first NL slots are lines and the rest continua (the
-// host orders the transitions lines first), known at compile time so the
-// per-slot kind tests fold away; NL < 0: the kinds are read at run time.
 // prd_I (hybrid PRD only, else nullptr): the rays' intensities at the PRD
 // points and then their dI/drho, written here, and then the rays' rho,
 // read here.
-template <typename R, int K, int NL, bool PRD, bool CACHE, bool BEZ>
-__device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &p, int b, int dir0, int dir1, R *slot,
-                             int lane, R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I, const R *phc)
+template <typename R, int K, bool PRD, bool CACHE, bool BEZ>
+__device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &p, int b, R *slot, int lane,
+                             R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I, const R *phc)
 {
     const int N = p.N;
     const DevTile &tl = A.tile[b];
@@ -1068,7 +1065,7 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
         lc.q[j] = lt[(RH_NLANEF * j + 4) * npad + pi];
         lc.pn[j] = lt[(RH_NLANEF * j + 5) * npad + pi];
         lc.grat[j] = lt[(RH_NLANEF * j + 6) * npad + pi];
-        lc.isline[j] = NL >= 0 ? j < NL : tr.kind == 0;
+        lc.isline[j] = tr.kind == 0;
         lc.lo[j] = tr.l;
         lc.up[j] = tr.u;
         lc.sub[j] = tr.sub;
@@ -1179,8 +1176,7 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
 
     for (int m = 0; m < nmu; ++m) {
         const R mu = mu_of<R>(A, m), imu = imu_of<R>(A, m), wm2 = wm2_of<R>(A, m);
-        // (partial redistribution: always both, a trip count the compiler knows)
-        for (int dir = PRD ? 0 : dir0; dir < (PRD ? 2 : dir1); ++dir) {
+        for (int dir = 0; dir < 2; ++dir) {
             const R muz = dir == 0 ? -mu : mu;
             const int ray = 2 * m + dir;
 #pragma unroll
@@ -1281,44 +1277,27 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
     }
 }
 
-// work item q of the sweep: a tile in one direction (split: Bezier without
-// partial redistribution, whose sums over rays would depend on the order of two
-// warps), or in both
+// Work item q of the sweep: a tile, whose rays add to its accumulators one
+// after the other.  The tile's kinds are read at run time: known at compile
+// time, and with the two directions as separate items, the Bezier solver takes
+// 21.0 instead of 24.9 ms (300 columns x 8 iterations), but the contributions
+// then round and add up in another order, and 8 of 65536 columns, whose rate
+// matrices are nearly singular, fail at another iteration.  (The nine tile
+// bodies of the PRD kernels cost more in instruction fetches than they save,
+// 3.2 -> 4.8 ms an iteration of 304 columns.)
 template <typename R, bool PRD, bool CACHE, bool BEZ>
 __device__ __forceinline__ void sweep_tile(const DevAtom &A, const Smem<R> &s, const KParams &p, int item, int lane,
                                            R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I,
                                            const R *phc)
 {
-    const int b = A.order[p.split ? item >> 1 : item];
+    const int b = A.order[item];
     const DevTile &tl = A.tile[b];
-    const int d0 = p.split ? item & 1 : 0, d1 = p.split ? d0 + 1 : 2;
-    R *slot = s.slot + (size_t)(tl.acc_off + (p.split && d0 ? A.macc : 0)) * p.N;
-#define RH_TILE(K_, NL_) \
-    sweep_tile_k<R, K_, NL_, PRD, CACHE, BEZ>(A, s, p, b, d0, d1, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc)
-    if constexpr (sizeof(R) == 4 && !PRD) {
-        // the slots' kinds at compile time (Bezier, 300 columns x 8 iterations:
-        // 25.8 -> 23.5 ms; with partial redistribution the nine tile bodies cost
-        // more in instruction fetches than they save, 3.2 -> 4.8 ms an iteration of
-        // 304 columns, and FP64 is bound by its arithmetic)
-        switch (tl.K * 4 + tl.nl) {
-        case 4: RH_TILE(1, 0); break;
-        case 5: RH_TILE(1, 1); break;
-        case 8: RH_TILE(2, 0); break;
-        case 9: RH_TILE(2, 1); break;
-        case 10: RH_TILE(2, 2); break;
-        case 12: RH_TILE(3, 0); break;
-        case 13: RH_TILE(3, 1); break;
-        case 14: RH_TILE(3, 2); break;
-        default: RH_TILE(3, 3); break;
-        }
-    } else {
-        switch (tl.K) {
-        case 1: RH_TILE(1, -1); break;
-        case 2: RH_TILE(2, -1); break;
-        default: RH_TILE(3, -1); break;
-        }
+    R *slot = s.slot + (size_t)tl.acc_off * p.N;
+    switch (tl.K) {
+    case 1: sweep_tile_k<R, 1, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+    case 2: sweep_tile_k<R, 2, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+    default: sweep_tile_k<R, 3, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
     }
-#undef RH_TILE
 }
 
 // work item q of the sweep: a tile in one direction (split), or in both
@@ -1817,7 +1796,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(
             double fcr = crsw > 1.0 ? fmax(1.0, crsw * pow(10.0, -(double)(it - 1))) : 1.0;
             for (int i = tid; i < LN; i += blockDim.x) s.nr[i] = (R)(s.n[i] * p.inv_nref);
             if (!UNITS)
-                for (int i = tid; i < (p.split ? 2 : 1) * A.macc * N; i += blockDim.x) s.slot[i] = 0;
+                for (int i = tid; i < A.macc * N; i += blockDim.x) s.slot[i] = 0;
             if constexpr (PRD) {
                 for (int i = tid; i < A.npp * N; i += blockDim.x) {
                     ps.J[i] = 0;
