@@ -49,26 +49,27 @@ struct Shape {
 };
 
 // The kernel for the atom and options, its shared memory with bw warps and
-// its resident blocks.  The linear solver's kernels of complete
-// redistribution take each tile's two directions as separate work items,
-// with their own accumulators, where that costs no resident block (the
-// accumulators are the largest part of the shared memory): twice the items
-// balance the warps (20 tiles on 8 warps: 3 rounds of both directions, 5 of
-// one): 1000 columns x 12 iterations 42 -> 20 ms, one column 6.4 -> 5.8 ms,
-// FP64 43.0 -> 42.4 ms.
+// its resident blocks.  The linear sweeps of complete redistribution take a
+// tile's two directions as separate work items: twice the items balance the
+// warps (20 tiles on 8 warps: 3 rounds of both directions, 5 of one).  FP32
+// with the cache always (the totals are kept apart in global memory and summed
+// in a fixed order); FP64, whose directions then have accumulators of their
+// own, where those cost no resident block (43.0 -> 42.4 ms; an accumulator
+// is the downward sum plus the upward one either way).  So no result depends
+// on the launch shape.
 cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool bez, int bw, Shape &s)
 {
-    const bool f32 = precision == 1, units = !A.nprd && !bez;
+    const bool f32 = precision == 1, crd = !A.nprd && !bez;
     if (A.nprd) s.fn = f32 ? (bez ? mali_kernel_prd32_bez() : mali_kernel_prd32()) : mali_kernel_prd64(bez);
     else if (bez) s.fn = mali_kernel_bez(precision);
     else if (f32) s.fn = mali_kernel_crd32(cache, A.nmu <= 2 ? 1 : (A.nmu <= 4 || A.nmu > 6 ? 2 : 3));
     else s.fn = mali_kernel_crd64(cache);
-    if (units)   // profile ring (FP32 with the cache) or ray states (FP64) per warp
+    if (crd)   // profile ring (FP32 with the cache) or ray states (FP64) per warp
         s.piece = f32 ? (cache ? kRingSlots * A.maxnl * A.nmu * kWarp * (int)sizeof(float) : 0)
                       : 3 * A.nmu * kWarp * (int)sizeof(double);
     s.nvp = s.piece ? (int)(kVtabBytes / s.piece) : 0;
     const int extra = s.piece && bw > s.nvp ? ((bw - s.nvp) * s.piece + kScratchUnit - 1) / kScratchUnit : 0;
-    for (int split = 0; split <= (units ? 1 : 0); ++split) {
+    for (int split = 0; split <= (crd && !f32 ? 1 : 0); ++split) {
         // accumulators (of both directions), or the rate-matrix entries summed in their place
         const int macc = std::max(split ? 2 * A.macc : A.macc, (f32 ? 2 : 1) * A.nent);
         const size_t sm = f32 ? smem_bytes<float>(A.nlev, N, 0, A.ncont, A.nline, macc, extra)
@@ -85,7 +86,7 @@ cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool be
         if (split && per < s.per_sm) break;
         s.sm = sm;
         s.per_sm = per;
-        s.split = split;
+        s.split = crd && f32 ? cache : split;
         s.slot_rows = macc;
     }
     return cudaSuccess;
@@ -104,8 +105,10 @@ int default_warps(const DevAtom &A, const IterLaunch &o, bool bez)
 
 void fill_k2(KParams &p)
 {
-    const float c[kNK2] = {1.0f,       -1.0f,       -1.4426950408889634f, 0.5f,          -1.0f / 6,    1.0f / 24,
-                           -1.0f / 120, 1.0f / 720, -1.0f / 5040,         1.0f / 40320, -1.0f / 362880};
+    // 1, -1; w_o / d and (1 - e^{-d}) / d as polynomials in d (sc_weights)
+    const float c[kNK2] = {1.0f,        -1.0f,        0.5f,        -1.0f / 6,   1.0f / 24,    -1.0f / 120,
+                           1.0f / 720,  -1.0f / 5040, 1.0f / 40320, -1.0f / 362880, 1.0f,     -0.5f,
+                           1.0f / 6,    -1.0f / 24,   1.0f / 120,  -1.0f / 720, 1.0f / 5040,  -1.0f / 40320};
     for (int i = 0; i < kNK2; ++i) {
         uint32_t u;
         memcpy(&u, &c[i], 4);
@@ -226,7 +229,8 @@ cudaError_t launch_mali_prealloc(const DevAtom &A, const ColumnArrays &c, const 
     KParams p = make_params(A, c, lane_tab, npad, vtab, nref, nghist, queue, o);
     // without a profile cache (callers that cannot allocate) the sweep
     // evaluates the profiles; partial redistribution always has the cache
-    const bool cache = p.phic || !A.nphi, bez = o.formal == 1;
+    // (the FP32 linear sweep keeps its totals there too, also of an atom without lines)
+    const bool bez = o.formal == 1, cache = p.phic || (!A.nphi && (o.precision == 0 || A.nprd || bez));
     if (!cache && A.nprd) {
         snprintf(err, errn, "the partial-redistribution kernel needs the profile cache");
         return cudaErrorInvalidValue;

@@ -2,20 +2,18 @@
 //
 // One thread block owns one column at a time and runs all of that column's
 // MALI iterations with the column's state in shared memory: populations
-// (FP64), collisional rates (FP64), per-depth atmosphere scalars, and the
-// rate accumulators.  When it takes a column, the block evaluates the line
+// (FP64), per-depth atmosphere scalars, and the rate accumulators.  When it takes a column, the block evaluates the line
 // profiles of every line slot, ray and depth (they do not depend on the
 // populations) into a per-block cache in global memory.  Per iteration:
-//   1. warps take 32-wavelength tiles of the grid, one direction at a time,
-//      from a block-local queue; each lane owns one wavelength and sweeps
-//      depth with every angle in one pass (linear short characteristics,
-//      intensity and local operator in registers, profiles read from the
-//      cache two depths ahead through shared memory); at every depth the lane
-//      sums its rays' terms and forms its contributions to the preconditioned
-//      rate matrix (Rybicki & Hummer 1992), the warp reduce-scatters them
-//      with shuffles, and one lane per value writes it to the tile's
-//      accumulator of that direction (sweep_unit; partial redistribution and
-//      the Bezier solver take one angle per pass, sweep_tile_k);
+//   1. warps take 32-wavelength tiles of the grid from a block-local queue;
+//      each lane owns one wavelength and sweeps depth (linear short
+//      characteristics; a tile and direction, all angles in one pass:
+//      sweep_pairs in FP32, sweep_unit in FP64; with partial redistribution or
+//      the Bezier solver a tile, one ray per pass: sweep_tile_k); at every
+//      depth the lane forms its contributions to the preconditioned rate
+//      matrix (Rybicki & Hummer 1992), the warp reduce-scatters them with
+//      shuffles, and one lane per value holds the total for the tile's
+//      accumulator;
 //   2. the block sums the accumulators into each depth's rate matrix (FP64)
 //      plus collisions, then one thread per depth solves the rate equations
 //      (FP64, scaled unknowns, partial pivoting);
@@ -26,6 +24,8 @@
 // formal solution and the rate terms (float or double); the rate matrix,
 // the solve and Ng are always FP64.
 #pragma once
+#include <type_traits>
+
 #include "rh15d_internal.h"
 #include "rh15d_math64.h"
 
@@ -34,11 +34,11 @@ namespace rh {
 namespace mali {
 
 constexpr int kWarp = 32;
-// Profile ring of the FP32 sweep with the profile cache: per warp, its tile's
-// cached line profiles (every angle of the unit's direction) at kRingSlots
-// depths -- the depth being swept and the next two -- copied from the cache
-// by cp.async, so the HBM latency of a profile read is covered by two depth
-// steps without holding the values in registers.
+// Profile ring of the FP32 linear sweep with the profile cache: per warp, its
+// tile's cached line profiles (every angle of the unit's direction) at
+// kRingSlots depths -- the depth being swept and the next two -- copied from
+// the cache by cp.async, so the HBM latency of a profile read is covered by
+// two depth steps without holding the values in registers.
 constexpr int kRingSlots = 3;
 constexpr int kScratchUnit = 2304;              // granularity of the layout's scratch region, bytes
 constexpr size_t kVtabBytes = sizeof(float4) * (RH_VT_N + 1);
@@ -47,7 +47,7 @@ constexpr int kRedDoubles = 5 * kNgLanes + 8;   // block reduction scratch
 
 // constants of the packed sweep (fill_k2): operands of packed instructions
 // come from the constant bank; as literals each use would be two moves
-enum K2 { K2_ONE, K2_NEG, K2_NLOG2E, K2_C0, kNK2 = K2_C0 + 8 };
+enum K2 { K2_ONE, K2_NEG, K2_WO, K2_E0 = K2_WO + 8, kNK2 = K2_E0 + 8 };
 
 struct KParams {
     int64_t ncol;
@@ -91,7 +91,7 @@ struct KParams {
     // only needed while the profiles are built), the others' behind the layout
     int piece, nvp;
     int slot_rows;                   // rows of the accumulator region
-    int split;                       // 1: a tile's two directions are separate units with their own accumulators
+    int split;                       // 1: a tile's two directions are separate work items
     unsigned long long k2[kNK2];     // constants of the packed sweep, both halves alike (K2)
 };
 
@@ -133,13 +133,15 @@ __host__ __device__ inline size_t prd_bytes(const DevAtom &A, int N)
 // Per-block profile cache: the line profile phi (Voigt H(a, v) times its
 // normalisation and 1/Doppler width, v including the ray's Doppler shift)
 // of every line slot, direction (0 down, 1 up), depth, angle and lane in R
-// (phi_block, phi_elem).  The profiles do
+// (phi_block, phi_ray).  The profiles do
 // not depend on the populations, so a column builds them once and every
 // iteration reads them back instead of evaluating the Voigt function.
+// Behind them, for the FP32 linear sweep, the warps' totals (pair_sums).
 template <typename R>
 __host__ __device__ inline size_t phic_bytes(const DevAtom &A, int N)
 {
-    const size_t r = sizeof(R) * (size_t)A.nphi * 2 * A.nmu * N * 32;
+    size_t r = sizeof(R) * (size_t)A.nphi * 2 * A.nmu * N * 32;
+    if (sizeof(R) == 4 && !A.nprd) r += sizeof(R) * (size_t)((A.nmu + 1) / 2 * 2) * A.macc * N;
     return (r + 255) & ~(size_t)255;
 }
 
@@ -260,13 +262,6 @@ __host__ __device__ size_t smem_bytes(int L, int N, int ntr, int ncont, int nlin
     return smem_layout<R>(L, N, ntr, ncont, nline, macc, ring_warps).end;
 }
 
-// sweeps that read the line profiles through the ring
-template <typename R, bool CACHE>
-__host__ __device__ constexpr bool uses_ring()
-{
-    return CACHE && sizeof(R) == 4;
-}
-
 template <typename R>
 __device__ Smem<R> carve(char *base, int L, int N, int ntr, int ncont, int nline, int macc, int ring_warps)
 {
@@ -339,9 +334,6 @@ __device__ __forceinline__ double line_phi(double q, double muz, double vz, doub
 template <typename R> __device__ __forceinline__ R rcp(R x);
 template <> __device__ __forceinline__ float rcp<float>(float x) { return rcp_f32(x); }
 template <> __device__ __forceinline__ double rcp<double>(double x) { return 1.0 / x; }
-
-__device__ __forceinline__ float rcp1(float x) { return rcp_f32(x); }
-__device__ __forceinline__ double rcp1(double x) { return rcp64(x); }
 
 // 1 - exp(-x) for x > 0: FP32 uses 1 - __expf(-x) (x = h nu / kT > 0.1 on every grid here,
 // relative error < 1e-6), FP64 expm1
@@ -489,117 +481,7 @@ template <int M> struct Pow2 { static constexpr int v = M <= 1 ? 1 : (M <= 2 ? 2
 template <int P> struct Log2 { static constexpr int v = P <= 1 ? 0 : 1 + Log2<P / 2>::v; };
 template <> struct Log2<1> { static constexpr int v = 0; };
 
-// ---- vectors of rays --------------------------------------------------------
-// The sweep's arithmetic runs on V = VecOf<R>: two FP32 values in a register
-// pair (two angles; one packed instruction does both, so the FP32 sweep, which
-// is bound by instruction issue, issues half as many), or one FP64 value.
-struct f2 {
-    unsigned long long u;
-};
-__device__ __forceinline__ f2 pk(float lo, float hi)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.u) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void upk(f2 a, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.u));
-}
-__device__ __forceinline__ f2 vfma(f2 a, f2 b, f2 c)
-{
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(a.u), "l"(b.u), "l"(c.u));
-    return r;
-}
-__device__ __forceinline__ f2 vmul(f2 a, f2 b)
-{
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
-    return r;
-}
-__device__ __forceinline__ f2 vadd(f2 a, f2 b)
-{
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
-    return r;
-}
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
-__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
-template <typename R> struct VecOf;
-template <> struct VecOf<float> {
-    typedef f2 V;
-    static constexpr int W = 2;
-    static __device__ __forceinline__ f2 splat(float x) { return pk(x, x); }
-};
-template <> struct VecOf<double> {
-    typedef double V;
-    static constexpr int W = 1;
-    static __device__ __forceinline__ double splat(double x) { return x; }
-};
-__device__ __forceinline__ float vsum(f2 a)
-{
-    float lo, hi;
-    upk(a, lo, hi);
-    return __fadd_rn(lo, hi);
-}
-__device__ __forceinline__ double vsum(double a) { return a; }
-__device__ __forceinline__ f2 vrcp(f2 a)
-{
-    float lo, hi;
-    upk(a, lo, hi);
-    return pk(rcp_f32(lo), rcp_f32(hi));
-}
-__device__ __forceinline__ double vrcp(double a) { return rcp64(a); }
-
-// Linear short-characteristics weights of a vector: e^{-d}, w_u, w_o and
-// 1 - w_o (see sc_weights).  Both forms are evaluated and selected per ray,
-// without a branch: the rays of a warp straddle d = 1/2 at most depths, and a
-// straight line of packed instructions costs less than the divergent branch
-// it replaces.  Below 1/2, p = (d - 1 + e^{-d}) / d^2 = sum (-d)^n / (n+2)!
-// (8 terms, truncation 2e-9) gives w_o = d p, 1 - e^{-d} = d (1 - w_o).
-__device__ __forceinline__ void vsc(const KParams &kp, f2 d, f2 &e, f2 &wu, f2 &wo, f2 &q)
-{
-    auto C = [&](int i) { return f2{kp.k2[i]}; };
-    const f2 one = C(K2_ONE), neg = C(K2_NEG);
-    f2 p = vfma(d, C(K2_C0 + 7), C(K2_C0 + 6));
-#pragma unroll
-    for (int i = 5; i >= 0; --i) p = vfma(p, d, C(K2_C0 + i));
-    const f2 wos = vmul(d, p), qs = vfma(wos, neg, one), e0 = vmul(d, qs);
-    const f2 wus = vfma(wos, neg, e0);
-    const f2 es = vfma(vmul(d, neg), qs, one);   // 1 - d q, rounded once
-    float d0, d1, x0, x1;
-    upk(d, d0, d1);
-    upk(vmul(d, C(K2_NLOG2E)), x0, x1);
-    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(x0));
-    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(x1));
-    const f2 ex = pk(x0, x1);
-    const f2 ql = vmul(vfma(ex, neg, one), pk(rcp_f32(d0), rcp_f32(d1)));
-    const f2 wol = vfma(ql, neg, one), wul = vfma(ex, neg, ql);
-    const bool s0 = d0 < 0.5f, s1 = d1 < 0.5f;
-    auto sel = [&](f2 a, f2 b) {
-        float a0, a1, b0, b1;
-        upk(a, a0, a1);
-        upk(b, b0, b1);
-        return pk(s0 ? a0 : b0, s1 ? a1 : b1);
-    };
-    e = sel(es, ex);
-    wu = sel(wus, wul);
-    wo = sel(wos, wol);
-    q = sel(qs, ql);
-}
-__device__ __forceinline__ void vsc(const KParams &kp, double d, double &e, double &wu, double &wo, double &q)
-{
-    sc64(d, kp.tab64, e, wu, wo, q);
-}
-
 // Planck terms of one wavelength at one depth: e^{-x}, 1 - e^{-x}
-__device__ __forceinline__ void planck_terms(float x, const double *, float &ex, float &om)
-{
-    ex = __expf(-x);
-    om = 1.0f - ex;
-}
 __device__ __forceinline__ void planck_terms(double x, const double *tab, double &ex, double &om)
 {
     if (x < 0.5) {   // 1 - e^{-x} by expm1 where it would cancel
@@ -611,16 +493,16 @@ __device__ __forceinline__ void planck_terms(double x, const double *tab, double
     }
 }
 
-// Element of the profile cache for cache row `row`, direction dir, depth k,
-// angle m and lane: [row][dir][depth] blocks of nmu x 32 values; PAIRS (the FP32
-// kernels of sweep_unit): two angles interleaved, the last of an odd number of
-// angles alone.  (int: at most 288 rows x 2 x 4096 depths x 8 angles x 32
+// First element of the profile cache for cache row `row`, direction dir and
+// depth k in the layout of the linear sweeps, [row][dir][depth] blocks of all
+// angles x 32 lanes.  (int: at most 288 rows x 2 x 4096 depths x 8 angles x 32
 // lanes < 2^31)
-template <typename R>
 __device__ __forceinline__ int phi_block(int nmu, int N, int row, int dir, int k)
 {
     return ((row * 2 + dir) * N + k) * (nmu * kWarp);
 }
+// ... and the element of an angle and lane in it; PAIRS (sweep_pairs): two
+// angles interleaved, the last of an odd number of angles alone
 template <bool PAIRS>
 __device__ __forceinline__ int phi_elem(int nmu, int m, int lane)
 {
@@ -637,32 +519,32 @@ __device__ __forceinline__ int phi_ray(int nmu, int N, int row, int dir, int m)
 
 // Depth-dependent, angle-independent quantities of one lane (NL lines first,
 // then NC continua).
-template <typename R, int K, int NL>
+template <int K, int NL>
 struct DepthV {
     static constexpr int NC = K - NL;
-    R chi0, eta0, etabg, B;             // background + continua; background; Planck function
-    R X[K], Rs[K];                      // n_l - R n_u, R
-    R A[NL ? NL : 1], El[NL ? NL : 1];  // line opacity and emissivity per profile
-    R Ut[NC ? NC : 1], oc[NC ? NC : 1]; // continuum U; opacity of the other continua and the background
+    double chi0, eta0, etabg, B;             // background + continua; background; Planck function
+    double X[K], Rs[K];                      // n_l - R n_u, R
+    double A[NL ? NL : 1], El[NL ? NL : 1];  // line opacity and emissivity per profile
+    double Ut[NC ? NC : 1], oc[NC ? NC : 1]; // continuum U; opacity of the other continua and the background
 };
 
-template <typename R, int K, int NL>
-__device__ __forceinline__ void depth_terms(const Smem<R> &s, const LaneC<R, K> &lc, const double *tab, int k, int N,
-                                            DepthV<R, K, NL> &d)
+template <int K, int NL>
+__device__ __forceinline__ void depth_terms(const Smem<double> &s, const LaneC<double, K> &lc, const double *tab, int k,
+                                            int N, DepthV<K, NL> &d)
 {
     constexpr int NC = K - NL;
-    R hkT, kff, nhm, thom, ex, om;
+    double hkT, kff, nhm, thom, ex, om;
     load4(s.bg + 4 * k, hkT, kff, nhm, thom);
     planck_terms(lc.nu * hkT, tab, ex, om);
-    const R chibg = (kff * lc.nu3s + nhm * lc.hm) * om + thom;
-    d.B = lc.tw * ex * rcp1(om);
+    const double chibg = (kff * lc.nu3s + nhm * lc.hm) * om + thom;
+    d.B = lc.tw * ex * rcp64(om);
     d.etabg = chibg * d.B;
     d.chi0 = chibg;
     d.eta0 = d.etabg;
-    R ch[NC ? NC : 1];
+    double ch[NC ? NC : 1];
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        const R nl = s.nr[lc.lo[j] * N + k], nu = s.nr[lc.up[j] * N + k];
+        const double nl = s.nr[lc.lo[j] * N + k], nu = s.nr[lc.up[j] * N + k];
         if (j < NL) {
             d.Rs[j] = lc.grat[j];
             d.X[j] = nl - d.Rs[j] * nu;
@@ -686,9 +568,9 @@ __device__ __forceinline__ void depth_terms(const Smem<R> &s, const LaneC<R, K> 
     }
 }
 
-// Sums over the rays of one depth, per vector element (w the ray's weight
-// w_mu/2, phi 1 for a continuum, Psi = Psi* per unit emissivity, q = 1 - Psi*
-// chi of the whole opacity, o_j the opacity of everything but transition j):
+// Sums over the rays of one depth (w the ray's weight w_mu/2, phi 1 for a
+// continuum, Psi = Psi* per unit emissivity, q = 1 - Psi* chi of the whole
+// opacity, o_j the opacity of everything but transition j):
 //   P_l = sum w phi_l I_eff, F_l = sum w phi_l (q + Psi o_l), S_l = sum w phi_l Psi (lines)
 //   T_ll' = sum w Psi phi_l phi_l'   (pairs of lines)
 //   Pc = sum w I_eff, Fc = sum w (q + Psi chi_lines), S0 = sum w Psi (shared by the continua:
@@ -697,39 +579,34 @@ __device__ __forceinline__ void depth_terms(const Smem<R> &s, const LaneC<R, K> 
 // the sums once per depth instead of every ray's terms; with
 //   up_j = c_j P_j, down_j = c_j R_j (E_j F_j + P_j), cross_jj' = c_j X_j U_j' (sum)
 // all terms of the sums are positive, nothing nearly equal is subtracted.
-template <typename V, int NL, int NC>
+// FP64 only: phi I_eff of a wing below a cold temperature minimum leaves the
+// FP32 range before c_j brings it back.
+template <int NL, int NC>
 struct RaySums {
     static constexpr int NT = NL * (NL - 1) / 2;
-    V P[NL ? NL : 1], F[NL ? NL : 1], S[NL ? NL : 1], T[NT ? NT : 1], Pc, Fc, S0;
+    double P[NL ? NL : 1], F[NL ? NL : 1], S[NL ? NL : 1], T[NT ? NT : 1], Pc, Fc, S0;
 };
 
-// One unit of the sweep: tile b (K transitions in its union, the first NL of
-// them lines) in one direction (dir 0 down, 1 up), every angle in one pass
+// One unit of the FP64 sweep: tile b (K transitions in its union, the first NL
+// of them lines) in one direction (dir 0 down, 1 up), every angle in one pass
 // over depth, so the depth terms and the warp's reductions are paid once per
 // depth and direction.  One lane = one wavelength.  At each depth the lane
 // forms the rays' sums above and from them its contributions to the
 // preconditioned rate matrix; the warp sums them over its wavelengths and
-// lane a writes accumulator a.  NV: vectors of rays per pass, held in
-// registers (FP32); 0: one ray at a time, the ray's state in shared memory
-// (FP64, where registers would not hold all rays).  The FP32 sweep is bound by
-// instruction issue: for 608 columns x 12 iterations (82 depths, 608
-// wavelengths, 5 angles) two angles per pass in scalar code took 15.9e9 warp
-// instructions and 21.3 ms, this 9.0e9 and 12.0 ms (62 % of the issue slots,
-// FMA pipe 42 %).  The FP64 sweep is bound by the FP64 pipe (150 columns x 3
-// iterations, profiles included: 371 -> 42 ms).  Atoms with more than 2 NV
-// angles take several passes (NV divides the number of vectors).
-template <typename R, int K, int NL, int NV, bool CACHE>
-__device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p, int b, int dir, R *slot, bool add0,
-                           int lane, const R *phc)
+// lane a writes accumulator a.  The rays' states are in the warp's shared
+// scratch (registers would not hold all rays).  Bound by the FP64 pipe (150
+// columns x 3 iterations, profiles included: 371 -> 42 ms against one angle
+// pair per pass with the library's exponentials and divisions).
+template <int K, int NL, bool CACHE>
+__device__ void sweep_unit(const DevAtom &A, const Smem<double> &s, const KParams &p, int b, int dir, double *slot,
+                           bool add, int lane, const double *phc)
 {
-    typedef typename VecOf<R>::V V;
-    constexpr int W = VecOf<R>::W, NC = K - NL, NVR = NV ? NV : 1;
-    auto splat = [](R x) { return VecOf<R>::splat(x); };
+    constexpr int NC = K - NL;
     const int N = p.N, nmu = A.nmu, npad = p.npad, pi = b * kWarp + lane;
     const DevTile &tl = A.tile[b];
-    const R *lt = reinterpret_cast<const R *>(p.lane);
+    const double *lt = reinterpret_cast<const double *>(p.lane);
     const double *tab = p.tab64;
-    LaneC<R, K> lc;
+    LaneC<double, K> lc;
     int poff[NL ? NL : 1];                       // first cache element of each line slot, this direction
 #pragma unroll
     for (int j = 0; j < K; ++j) {
@@ -744,7 +621,7 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p,
         }
         if (j < NL) {
             lc.grat[j] = lt[(RH_NLANEF * j + 6) * npad + pi];
-            poff[j] = CACHE ? phi_block<R>(nmu, N, tl.phi[j], dir, 0) : 0;
+            poff[j] = CACHE ? phi_block(nmu, N, tl.phi[j], dir, 0) : 0;
         }
         lc.lo[j] = tr.l;
         lc.up[j] = tr.u;
@@ -760,304 +637,192 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<R> &s, const KParams &p,
     constexpr int SH = 5 - Log2<P>::v;
     const bool writer = (lane & ((1 << SH) - 1)) == 0;
     const int widx = lane >> SH;
-    const int nvec = (nmu + W - 1) / W;          // vectors of rays, the last maybe with a padding ray of weight 0
-    constexpr bool RING = uses_ring<R, CACHE>() && NL > 0;
-    // the warp's shared scratch: profile ring (RING) or ray states (NV = 0)
-    R *wscr = reinterpret_cast<R *>(warp_scratch(s, p, threadIdx.x >> 5));
+    // ray m's I, chi and S of the upwind point at st[0], st[kWarp], st[2 kWarp]
+    double *rays = reinterpret_cast<double *>(warp_scratch(s, p, threadIdx.x >> 5)) + lane;
     const int blk = nmu * kWarp;
 
-    for (int v0 = 0; v0 < nvec; v0 += NV ? NV : nvec) {
-        V mw[NVR], imu[NVR];                     // weights, 1/(2 mu) of the pass's rays
-        if constexpr (NV > 0) {
+    auto phi_at = [&](int j, int m, int k) -> double {
+        if constexpr (CACHE) return phc[poff[j] + k * blk + phi_elem<false>(nmu, m, lane)];
+        else
+            return line_phi(lc.q[j], dir ? A.mu[m] : -A.mu[m], s.vz[k], s.ivth[k], s.ad[lc.sub[j] * N + k], lc.pn[j],
+                            s.vtab, tab);
+    };
+    RaySums<NL, NC> rs;
+    auto zero = [&]() {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const int m = 2 * (v0 + v), m2 = m + 1 < nmu ? m + 1 : m;
-                mw[v] = pk(A.wm2f[m], m + 1 < nmu ? A.wm2f[m2] : 0.0f);
-                imu[v] = pk(0.5f * A.imuf[m], 0.5f * A.imuf[m2]);
-            }
-        }
-        // profiles of vector v (of the pass) of line slot j at depth k, straight from the cache or evaluated
-        auto phi_at = [&](int j, int v, int k) -> V {
-            if constexpr (W == 2) {
-                const int m1 = 2 * (v0 + v), m2 = m1 + 1 < nmu ? m1 + 1 : m1;
-                if constexpr (CACHE) {
-                    const R *c = phc + poff[j] + k * blk;
-                    return pk(c[phi_elem<sizeof(R) == 4>(nmu, m1, lane)], c[phi_elem<sizeof(R) == 4>(nmu, m2, lane)]);
-                } else {
-                    const R a = s.ad[lc.sub[j] * N + k], z1 = dir ? A.muf[m1] : -A.muf[m1],
-                            z2 = dir ? A.muf[m2] : -A.muf[m2];
-                    return pk(line_phi(lc.q[j], z1, s.vz[k], s.ivth[k], a, lc.pn[j], s.vtab, tab),
-                              line_phi(lc.q[j], z2, s.vz[k], s.ivth[k], a, lc.pn[j], s.vtab, tab));
-                }
-            } else {
-                const int m = v0 + v;
-                if constexpr (CACHE) return phc[poff[j] + k * blk + phi_elem<sizeof(R) == 4>(nmu, m, lane)];
-                else
-                    return line_phi(lc.q[j], dir ? A.mu[m] : -A.mu[m], s.vz[k], s.ivth[k], s.ad[lc.sub[j] * N + k],
-                                    lc.pn[j], s.vtab, tab);
-            }
-        };
-        RaySums<V, NL, NC> rs;
-        auto zero = [&]() {
-            const V z = splat((R)0);
+        for (int j = 0; j < NL; ++j) rs.P[j] = rs.F[j] = rs.S[j] = 0.0;
 #pragma unroll
-            for (int j = 0; j < NL; ++j) rs.P[j] = rs.F[j] = rs.S[j] = z;
-#pragma unroll
-            for (int j = 0; j < RaySums<V, NL, NC>::NT; ++j) rs.T[j] = z;
-            rs.Pc = rs.Fc = rs.S0 = z;
-        };
-        // opacity and emissivity of a vector of rays; ls: the lines' part of the opacity
-        auto opac = [&](const DepthV<R, K, NL> &d, const V (&ph)[NL ? NL : 1], V &chi, V &eta, V &ls) {
-            eta = splat(d.eta0);
-            if constexpr (NL == 0) {
-                chi = splat(d.chi0);
-            } else {
-                if constexpr (NC > 0 || NL > 1) {
-                    ls = vmul(splat(d.A[0]), ph[0]);
-#pragma unroll
-                    for (int j = 1; j < NL; ++j) ls = vfma(splat(d.A[j]), ph[j], ls);
-                    chi = NL == 1 ? vfma(splat(d.A[0]), ph[0], splat(d.chi0)) : vadd(splat(d.chi0), ls);
-                } else {
-                    chi = vfma(splat(d.A[0]), ph[0], splat(d.chi0));
-                }
-#pragma unroll
-                for (int j = 0; j < NL; ++j) eta = vfma(splat(d.El[j]), ph[j], eta);
-            }
-        };
-        // a vector's terms of the sums
-        // (first: the depth's first vector starts the sums)
-        auto accumulate = [&](const DepthV<R, K, NL> &d, const V (&ph)[NL ? NL : 1], V w, V ls, V q, V psi, V Ieff,
-                              bool first) {
-            auto sum = [&](V &acc, V a, V b) { acc = first ? vmul(a, b) : vfma(a, b, acc); };
-            if constexpr (NC > 0) {
-                sum(rs.Pc, w, Ieff);
-                sum(rs.Fc, w, NL > 0 ? vfma(psi, ls, q) : q);
-                sum(rs.S0, w, psi);
-            }
-#pragma unroll
-            for (int j = 0; j < NL; ++j) {
-                const V wp = vmul(w, ph[j]);
-                V o = splat(d.chi0);
-                int t = 0;
-#pragma unroll
-                for (int a = 0; a < NL; ++a)
-#pragma unroll
-                    for (int c = a + 1; c < NL; ++c, ++t) {
-                        if (a == j) o = vfma(splat(d.A[c]), ph[c], o);
-                        if (c == j) o = vfma(splat(d.A[a]), ph[a], o);
-                        if (a == j) sum(rs.T[t], vmul(wp, psi), ph[c]);
-                    }
-                sum(rs.P[j], wp, Ieff);
-                sum(rs.F[j], wp, vfma(psi, o, q));
-                if constexpr (NC > 0) sum(rs.S[j], wp, psi);
-            }
-        };
-        // the lane's contributions from the sums, summed over the warp
-        auto flush = [&](const DepthV<R, K, NL> &d, int k) {
-            R val[P], Pj[K], S[NL ? NL : 1];
-#pragma unroll
-            for (int a = M; a < P; ++a) val[a] = 0;
-            const R Pc = NC ? vsum(rs.Pc) : (R)0, Fc = NC ? vsum(rs.Fc) : (R)0, S0 = NC ? vsum(rs.S0) : (R)0;
-#pragma unroll
-            for (int j = 0; j < K; ++j) {
-                R Fj;
-                if (j < NL) {
-                    Pj[j] = vsum(rs.P[j]);
-                    Fj = vsum(rs.F[j]);
-                    if (NC) S[j] = vsum(rs.S[j]);
-                } else {
-                    Pj[j] = Pc;
-                    Fj = Fc + d.oc[j - NL] * S0;
-                }
-                val[j] = lc.c[j] * Pj[j];
-                val[K + j] = lc.c[j] * d.Rs[j] * (lc.E[j] * Fj + Pj[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < K; ++j)
-#pragma unroll
-                for (int j2 = 0; j2 < K; ++j2) {
-                    if (j2 == j) continue;
-                    const int lo = j < j2 ? j : j2, hi = j < j2 ? j2 : j;
-                    R x;
-                    if (hi < NL) x = vsum(rs.T[lo * NL - lo * (lo + 1) / 2 + hi - lo - 1]);
-                    else if (lo < NL) x = S[lo];
-                    else x = S0;
-                    const R u = j2 < NL ? lc.Uc[j2] : d.Ut[j2 - NL < 0 ? 0 : j2 - NL];
-                    // the sum first: c X U alone can leave the FP32 range
-                    val[2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1)] = lc.c[j] * x * d.X[j] * u;
-                }
-            const R t = reduce_scatter<P>(val, lane);
-            if (writer && widx < M) {
-                R *o = slot + widx * N + k;
-                *o = (add0 || v0 > 0) ? *o + t : t;
-            }
-        };
-        // ---- boundary point: I = 0 at the top; at the bottom the diffusion
-        // condition, which needs chi and B one point up
-        const int k0 = dir == 0 ? 0 : N - 1;
-        V I[NVR], chip[NVR], Sp[NVR];
-        DepthV<R, K, NL> d2, d;
-        if (dir == 1) depth_terms<R, K, NL>(s, lc, tab, N - 2, N, d2);
-        depth_terms<R, K, NL>(s, lc, tab, k0, N, d);
-        if constexpr (NV == 0) zero();
-        auto boundary = [&](int v, V w, V im, V &Iv, V &chv, V &Sv) {
-            V ph[NL ? NL : 1], chi, eta, ls = splat((R)0), ch2 = splat((R)0);
-            if (dir == 1) {
-#pragma unroll
-                for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, v, N - 2);
-                opac(d2, ph, ch2, eta, ls);
-            }
-#pragma unroll
-            for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, v, k0);
-            opac(d, ph, chi, eta, ls);
-            const V ic = vrcp(chi);
-            Iv = splat((R)0);
-            if (dir == 1)   // B + mu (B - B2) / dtau = B + (B - B2) / (dtau / mu)
-                Iv = vfma(splat(d.B - d2.B), vrcp(vmul(vmul(vadd(chi, ch2), splat(s.dz[N - 2])), im)),
-                          splat(d.B));
-            chv = chi;
-            Sv = vmul(eta, ic);
-            accumulate(d, ph, w, ls, splat((R)1), splat((R)0), Iv, NV > 0 && v == 0);
-        };
-        if constexpr (NV > 0) {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) boundary(v, mw[v], imu[v], I[v], chip[v], Sp[v]);
+        for (int j = 0; j < RaySums<NL, NC>::NT; ++j) rs.T[j] = 0.0;
+        rs.Pc = rs.Fc = rs.S0 = 0.0;
+    };
+    // opacity and emissivity of a ray; ls: the lines' part of the opacity
+    auto opac = [&](const DepthV<K, NL> &d, const double (&ph)[NL ? NL : 1], double &chi, double &eta, double &ls) {
+        eta = d.eta0;
+        if constexpr (NL == 0) {
+            chi = d.chi0;
         } else {
-            for (int v = 0; v < nvec; ++v) {
-                V Iv, cv, Sv;
-                boundary(v, wm2_of<R>(A, v), (R)0.5 * imu_of<R>(A, v), Iv, cv, Sv);
-                R *st = wscr + (size_t)v * 3 * kWarp + lane;
-                st[0] = Iv;
-                st[kWarp] = cv;
-                st[2 * kWarp] = Sv;
-            }
-        }
-        flush(d, k0);
-        // one step of a vector of rays to depth k
-        auto step_ray = [&](const V (&ph)[NL ? NL : 1], V w, V hz, V &Iv, V &chv, V &Sv, bool first) {
-            V chi, eta, ls = splat((R)0), e, wu, wo, q;
-            opac(d, ph, chi, eta, ls);
-            const V ic = vrcp(chi), S = vmul(eta, ic);
-            vsc(p, vmul(vadd(chi, chv), hz), e, wu, wo, q);
-            const V base = vfma(Iv, e, vmul(wu, Sv)), psi = vmul(wo, ic);
-            Iv = vfma(wo, S, base);
-            chv = chi;
-            Sv = S;
-            accumulate(d, ph, w, ls, q, psi, vfma(psi, splat(d.etabg), base), first);
-        };
-        // profile ring: the copies of step st's depth go into slot st mod 3,
-        // issued two steps ahead (one commit group per step, empty past the end)
-        const int rstride = A.maxnl * blk, gstep = dir == 0 ? blk : -blk;
-        const R *src = phc;                      // this lane's first element of the next depth to copy
-        int fst = 1, foff = rstride, roff = rstride;   // its step, its ring offset; the offset being read
-        if constexpr (RING) src = phc + (dir == 0 ? 1 : N - 2) * blk + 4 * lane;
-        auto ring_fill = [&]() {
-            if constexpr (RING) {
-                if (fst < N) {
-                    R *dst = wscr + foff + 4 * lane;
+            if constexpr (NC > 0 || NL > 1) {
+                ls = d.A[0] * ph[0];
 #pragma unroll
-                    for (int j = 0; j < NL; ++j) {   // nmu x 32 values: at most two 16-byte pieces a lane
-                        if (lane < nmu * 8) cp_async16(dst + j * blk, src + poff[j]);
-                        if (lane + kWarp < nmu * 8) cp_async16(dst + j * blk + 4 * kWarp, src + poff[j] + 4 * kWarp);
-                    }
-                }
-                cp_async_commit();
-                ++fst;
-                src += gstep;
-                foff = foff == 2 * rstride ? 0 : foff + rstride;
-            }
-        };
-        ring_fill();
-        ring_fill();
-        for (int st = 1; st < N; ++st) {
-            const int k = dir == 0 ? st : N - 1 - st;
-            const R *rg = nullptr;
-            if constexpr (RING) {
-                cp_async_wait<1>();
-                __syncwarp();
-                rg = wscr + roff;
-                ring_fill();   // into the slot read one step ago
-                roff = roff == 2 * rstride ? 0 : roff + rstride;
-            }
-            depth_terms<R, K, NL>(s, lc, tab, k, N, d);
-            const R dzk = dir == 0 ? s.dz[k - 1] : s.dz[k];
-            if constexpr (NV == 0) zero();
-            if constexpr (NV > 0) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    V ph[NL ? NL : 1];
-#pragma unroll
-                    for (int j = 0; j < NL; ++j) {
-                        if constexpr (RING) {
-                            const int m = 2 * (v0 + v);
-                            const R *r = rg + j * blk + m * kWarp;
-                            // a full pair in one read; the last vector's lone angle fills both halves
-                            if (v < NV - 1) {
-                                ph[j].u = *reinterpret_cast<const unsigned long long *>(r + 2 * lane);
-                            } else {
-                                const bool full = m + 1 < nmu;
-                                const R lo = r[full ? 2 * lane : lane], hi = full ? r[2 * lane + 1] : lo;
-                                ph[j] = pk(lo, hi);
-                            }
-                        } else {
-                            ph[j] = phi_at(j, v, k);
-                        }
-                    }
-                    step_ray(ph, mw[v], vmul(imu[v], splat(dzk)), I[v], chip[v], Sp[v], v == 0);
-                }
+                for (int j = 1; j < NL; ++j) ls = fma(d.A[j], ph[j], ls);
+                chi = NL == 1 ? fma(d.A[0], ph[0], d.chi0) : d.chi0 + ls;
             } else {
-                for (int v = 0; v < nvec; ++v) {
-                    V ph[NL ? NL : 1];
-#pragma unroll
-                    for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, v, k);
-                    R *sp = wscr + (size_t)v * 3 * kWarp + lane;
-                    V Iv = sp[0], cv = sp[kWarp], Sv = sp[2 * kWarp];
-                    step_ray(ph, wm2_of<R>(A, v), (R)0.5 * imu_of<R>(A, v) * dzk, Iv, cv, Sv, false);
-                    sp[0] = Iv;
-                    sp[kWarp] = cv;
-                    sp[2 * kWarp] = Sv;
-                }
+                chi = fma(d.A[0], ph[0], d.chi0);
             }
-            flush(d, k);
+#pragma unroll
+            for (int j = 0; j < NL; ++j) eta = fma(d.El[j], ph[j], eta);
         }
-        if constexpr (RING) {
-            cp_async_wait<0>();
-            __syncwarp();
+    };
+    // a ray's terms of the sums
+    auto accumulate = [&](const DepthV<K, NL> &d, const double (&ph)[NL ? NL : 1], double w, double ls, double q,
+                          double psi, double Ieff) {
+        if constexpr (NC > 0) {
+            rs.Pc = fma(w, Ieff, rs.Pc);
+            rs.Fc = fma(w, NL > 0 ? fma(psi, ls, q) : q, rs.Fc);
+            rs.S0 = fma(w, psi, rs.S0);
         }
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            const double wp = w * ph[j];
+            double o = d.chi0;
+            int t = 0;
+#pragma unroll
+            for (int a = 0; a < NL; ++a)
+#pragma unroll
+                for (int c = a + 1; c < NL; ++c, ++t) {
+                    if (a == j) o = fma(d.A[c], ph[c], o);
+                    if (c == j) o = fma(d.A[a], ph[a], o);
+                    if (a == j) rs.T[t] = fma(wp * psi, ph[c], rs.T[t]);
+                }
+            rs.P[j] = fma(wp, Ieff, rs.P[j]);
+            rs.F[j] = fma(wp, fma(psi, o, q), rs.F[j]);
+            if constexpr (NC > 0) rs.S[j] = fma(wp, psi, rs.S[j]);
+        }
+    };
+    // the lane's contributions from the sums, summed over the warp
+    auto flush = [&](const DepthV<K, NL> &d, int k) {
+        double val[P], Pj[K];
+#pragma unroll
+        for (int a = M; a < P; ++a) val[a] = 0;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            double Fj;
+            if (j < NL) {
+                Pj[j] = rs.P[j];
+                Fj = rs.F[j];
+            } else {
+                Pj[j] = rs.Pc;
+                Fj = rs.Fc + d.oc[j - NL] * rs.S0;
+            }
+            val[j] = lc.c[j] * Pj[j];
+            val[K + j] = lc.c[j] * d.Rs[j] * (lc.E[j] * Fj + Pj[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+#pragma unroll
+            for (int j2 = 0; j2 < K; ++j2) {
+                if (j2 == j) continue;
+                const int lo = j < j2 ? j : j2, hi = j < j2 ? j2 : j;
+                double x;
+                if (hi < NL) x = rs.T[lo * NL - lo * (lo + 1) / 2 + hi - lo - 1];
+                else if (lo < NL) x = rs.S[lo];
+                else x = rs.S0;
+                const double u = j2 < NL ? lc.Uc[j2] : d.Ut[j2 - NL < 0 ? 0 : j2 - NL];
+                val[2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1)] = lc.c[j] * x * d.X[j] * u;
+            }
+        const double t = reduce_scatter<P>(val, lane);
+        if (writer && widx < M) {
+            double *o = slot + widx * N + k;
+            *o = add ? *o + t : t;
+        }
+    };
+    // ---- boundary point: I = 0 at the top; at the bottom the diffusion
+    // condition, which needs chi and B one point up
+    const int k0 = dir == 0 ? 0 : N - 1;
+    DepthV<K, NL> d2, d;
+    if (dir == 1) depth_terms<K, NL>(s, lc, tab, N - 2, N, d2);
+    depth_terms<K, NL>(s, lc, tab, k0, N, d);
+    zero();
+    for (int m = 0; m < nmu; ++m) {
+        double ph[NL ? NL : 1], chi, eta, ls = 0.0, ch2 = 0.0, I = 0.0;
+        if (dir == 1) {
+#pragma unroll
+            for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, m, N - 2);
+            opac(d2, ph, ch2, eta, ls);
+        }
+#pragma unroll
+        for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, m, k0);
+        opac(d, ph, chi, eta, ls);
+        if (dir == 1)   // B + mu (B - B2) / dtau = B + (B - B2) / (dtau / mu)
+            I = fma(d.B - d2.B, rcp64((chi + ch2) * s.dz[N - 2] * (0.5 * A.imu[m])), d.B);
+        double *st = rays + (size_t)m * 3 * kWarp;
+        st[0] = I;
+        st[kWarp] = chi;
+        st[2 * kWarp] = eta * rcp64(chi);
+        accumulate(d, ph, wm2_of<double>(A, m), ls, 1.0, 0.0, I);
+    }
+    flush(d, k0);
+    for (int step = 1; step < N; ++step) {
+        const int k = dir == 0 ? step : N - 1 - step;
+        depth_terms<K, NL>(s, lc, tab, k, N, d);
+        const double dzk = dir == 0 ? s.dz[k - 1] : s.dz[k];
+        zero();
+        for (int m = 0; m < nmu; ++m) {
+            double ph[NL ? NL : 1];
+#pragma unroll
+            for (int j = 0; j < NL; ++j) ph[j] = phi_at(j, m, k);
+            double *st = rays + (size_t)m * 3 * kWarp;
+            double chi, eta, ls = 0.0, e, wu, wo, q;
+            opac(d, ph, chi, eta, ls);
+            const double ic = rcp64(chi), S = eta * ic;
+            sc64((chi + st[kWarp]) * (0.5 * A.imu[m] * dzk), tab, e, wu, wo, q);
+            const double base = fma(st[0], e, wu * st[2 * kWarp]), psi = wo * ic;
+            st[0] = fma(wo, S, base);
+            st[kWarp] = chi;
+            st[2 * kWarp] = S;
+            accumulate(d, ph, wm2_of<double>(A, m), ls, q, psi, fma(psi, d.etabg, base));
+        }
+        flush(d, k);
     }
 }
 
-// Sweep one tile (K transitions in its union) for every angle, downward and
-// upward, adding its rate accumulators.  One lane = one wavelength; the
-// angle loop runs outside the depth sweep so the lane state is scalar.  At
-// each depth the lane forms, without subtracting nearly equal numbers,
-//   I_eff = I - Psi* eta_active = I_u e^{-dtau} + w_u S_u + w_o eta_bg/chi,
-//   1 - Psi* chi_j = (1 - w_o) + w_o (chi - chi_j)/chi,
-// and its contributions (weight w = w_mu/2):
-//   up_j = c_j w phi_j I_eff,  down_j = c_j R_j w phi_j (E_j (1 - Psi* chi_j) + I_eff),
-//   cross_{j,j'} = c_j X_j w phi_j Psi* U_j';
-// the warp sums them over its wavelengths and lane a adds accumulator a.
-// PRD: the tile's PRD slot emits with psi = rho phi (rho of the lane's point
-// and depth from the block's scratch), PRD lanes accumulate the angle-averaged
-// mean intensity J, and every slot also accumulates its plain rates (actual
-// intensity) cw I and cw R (E + I), for the PRD update.
-// prd_I (hybrid PRD only, else nullptr): the rays' intensities at the PRD
-// points and then their dI/drho, written here, and then the rays' rho,
-// read here.
-template <typename R, int K, bool PRD, bool CACHE, bool BEZ>
-__device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &p, int b, R *slot, int lane,
-                             R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I, const R *phc)
+// Rate contributions of one ray at one depth point (add: accumulate into
+// val); see sweep_pairs.
+template <typename R, int K, int P>
+__device__ __forceinline__ void ray_rates(const LaneC<R, K> &lc, const DepthC<R, K> &d, const R (&phi)[K],
+                                          const R (&chj)[K], const R (&U)[K], R ichi, R wo, R omwo, R psi, R Ieff,
+                                          R wm2, R (&val)[P], bool add)
 {
-    const int N = p.N;
-    const DevTile &tl = A.tile[b];
-    const int nmu = A.nmu;
-    const R *lt = reinterpret_cast<const R *>(p.lane);
-    const int npad = p.npad;
-    const int pi = b * kWarp + lane;
-    LaneC<R, K> lc;
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        const DevTrans &tr = A.tr[tl.t[j]];
+        R other = d.chibg;
+#pragma unroll
+        for (int j2 = 0; j2 < K; ++j2)
+            if (j2 != j) other += chj[j2];
+        const R f = omwo + wo * other * ichi;          // 1 - Psi* chi_j
+        const R cw = lc.c[j] * wm2 * phi[j];
+        const R v0 = cw * Ieff, v1 = cw * d.Rs[j] * (lc.E[j] * f + Ieff);
+        val[j] = add ? val[j] + v0 : v0;
+        val[K + j] = add ? val[K + j] + v1 : v1;
+        const R cx = cw * d.Xs[j] * psi;
+#pragma unroll
+        for (int j2 = 0; j2 < K; ++j2)
+            if (j2 != j) {
+                const int a = 2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1);
+                val[a] = add ? val[a] + cx * U[j2] : cx * U[j2];
+            }
+    }
+}
+
+// Per-lane constants of tile b
+template <typename R, int K>
+__device__ __forceinline__ void load_lane(const DevAtom &A, const KParams &p, int b, int lane, LaneC<R, K> &lc)
+{
+    const R *lt = reinterpret_cast<const R *>(p.lane);
+    const int npad = p.npad, pi = b * kWarp + lane;
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const DevTrans &tr = A.tr[A.tile[b].t[j]];
         lc.c[j] = lt[(RH_NLANEF * j + 0) * npad + pi];
         lc.Vc[j] = lt[(RH_NLANEF * j + 1) * npad + pi];
         lc.Uc[j] = lt[(RH_NLANEF * j + 2) * npad + pi];
@@ -1074,22 +839,426 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
     lc.hm = lt[kLaneHm * npad + pi];
     lc.nu3s = lt[kLaneNu3 * npad + pi];
     lc.tw = lt[kLaneTw * npad + pi];
-    // line profiles of depth k, ray r (2 m + d) for the tile's line slots (0
-    // elsewhere): read from the column's cache (CACHE), or evaluated here (the
-    // same arithmetic as the cache's build)
-    int pb[K];                                     // the ray's first element of each line slot's cache rows
-    auto load_ph = [&](int k, int r, R (&o)[K]) {
+}
+
+// ---- the FP32 linear sweep ---------------------------------------------------
+// Two rays (two angles) in a register pair: one packed instruction does both,
+// so the sweep, which is bound by instruction issue, issues half as many.
+// Each half rounds as the scalar operation would.
+struct f2 {
+    unsigned long long u;
+};
+__device__ __forceinline__ f2 pk(float lo, float hi)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.u) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f2 splat(float x) { return pk(x, x); }
+__device__ __forceinline__ void upk(f2 a, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.u));
+}
+__device__ __forceinline__ f2 vfma(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(a.u), "l"(b.u), "l"(c.u));
+    return r;
+}
+__device__ __forceinline__ f2 vmul(f2 a, f2 b)
+{
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+    return r;
+}
+__device__ __forceinline__ f2 vadd(f2 a, f2 b)
+{
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+    return r;
+}
+// A product that keeps its rounding: the assembler fuses a packed product into
+// a packed sum that is its only use, in spite of both instructions' .rn; it
+// leaves scalar products alone.
+__device__ __forceinline__ f2 vmul_rn(f2 a, f2 b)
+{
+    float a0, a1, b0, b1;
+    upk(a, a0, a1);
+    upk(b, b0, b1);
+    return pk(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ f2 vrcp(f2 a)
+{
+    float lo, hi;
+    upk(a, lo, hi);
+    return pk(rcp_f32(lo), rcp_f32(hi));
+}
+
+// Linear short-characteristics weights of a pair, e^{-d}, w_u, w_o and 1 -
+// w_o, to the bit those of sc_weights.  Both of its forms are evaluated and
+// selected per ray, without a branch: the rays of a warp straddle d = 1/2 at
+// most depths, and a straight line of packed instructions costs less than the
+// divergent branch.
+__device__ __forceinline__ void vsc(const KParams &kp, f2 d, f2 &e, f2 &wu, f2 &wo, f2 &omwo)
+{
+    auto C = [&](int i) { return f2{kp.k2[i]}; };
+    const f2 one = C(K2_ONE), neg = C(K2_NEG), nd = vmul(d, neg);
+    f2 w = C(K2_WO + 7), q = C(K2_E0 + 7);
+#pragma unroll
+    for (int i = 6; i >= 0; --i) {
+        w = vfma(d, w, C(K2_WO + i));
+        q = vfma(d, q, C(K2_E0 + i));
+    }
+    const f2 wos = vmul(w, d), nwo = vmul_rn(w, nd), wus = vfma(d, q, nwo), oms = vadd(nwo, one), es = vfma(nd, q, one);
+    float d0, d1;
+    upk(d, d0, d1);
+    const f2 ex = pk(__expf(-d0), __expf(-d1));
+    const f2 oml = vmul(vfma(ex, neg, one), pk(rcp_f32(d0), rcp_f32(d1)));
+    const f2 wol = vfma(oml, neg, one), wul = vfma(ex, neg, oml);
+    const bool s0 = d0 < 0.5f, s1 = d1 < 0.5f;
+    auto sel = [&](f2 a, f2 b) {
+        float a0, a1, b0, b1;
+        upk(a, a0, a1);
+        upk(b, b0, b1);
+        return pk(s0 ? a0 : b0, s1 ? a1 : b1);
+    };
+    e = sel(es, ex);
+    wu = sel(wus, wul);
+    wo = sel(wos, wol);
+    omwo = sel(oms, oml);
+}
+
+// Where the sums of opacities round a transition's opacity on its own (bit j:
+// slot j) instead of fusing its last product into the sum: in chi and in the
+// opacity of the other transitions at a depth step, in chi at the first point
+// of a ray and at the point next to it that the diffusion condition reads; and
+// whether the emissivity at the first point fuses chi_bg B.  Any choice is as
+// accurate; these are kept because they have always been these kernels' (see
+// sweep_pairs).
+template <int K, int NL>
+struct Unfused {
+    static constexpr int step = K == 2 ? 2 : K == 3 && NL == 3 ? 6 : K == 3 && NL == 2 ? 2 : 0;
+    static constexpr int other = K == 2 && NL == 0 ? 0 : step;
+    static constexpr int first = K == 3 ? 6 : K == 2 ? 2 : 0;
+    static constexpr int next = K == 2 && NL == 0 ? 0 : K == 3 && NL == 1 ? 6 : step;
+    static constexpr bool eta_first = NL == 0;
+};
+
+// Depth-dependent, angle-independent quantities of one lane (the first NL
+// transitions lines, the others continua)
+template <int K>
+struct DepthF {
+    float chibg, etabg, B, etac;
+    float Rs[K], X[K], nu[K], chc[K], Uct[K];   // R, n_l - R n_u, n_u, continuum opacity, continuum U
+};
+template <int K, int NL>
+__device__ __forceinline__ void depth_f(const Smem<float> &s, const LaneC<float, K> &lc, int k, int N, DepthF<K> &d)
+{
+    float hkT, kff, nhm, thom;
+    load4(s.bg + 4 * k, hkT, kff, nhm, thom);
+    const float ex = __expf(-__fmul_rn(lc.nu, hkT)), om = __fsub_rn(1.0f, ex);   // h nu / kT > 0.1 on every grid
+    d.chibg = __fmaf_rn(__fmaf_rn(kff, lc.nu3s, __fmul_rn(nhm, lc.hm)), om, thom);
+    d.B = __fmul_rn(__fmul_rn(lc.tw, ex), rcp_f32(om));
+    d.etabg = __fmul_rn(d.chibg, d.B);
+    d.etac = 0.0f;
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const float nl = s.nr[lc.lo[j] * N + k];
+        d.nu[j] = s.nr[lc.up[j] * N + k];
+        d.Rs[j] = j < NL ? lc.grat[j] : __fmul_rn(s.Gc[lc.sub[j] * N + k], ex);
+        d.X[j] = __fmaf_rn(-d.Rs[j], d.nu[j], nl);
+        if (j >= NL) {
+            d.chc[j] = __fmul_rn(lc.Vc[j], d.X[j]);
+            d.Uct[j] = __fmul_rn(lc.Uc[j], d.Rs[j]);
+            d.etac = __fmaf_rn(d.nu[j], d.Uct[j], d.etac);
+        }
+    }
+}
+
+// The FP32 sweep of tile b (K transitions in its union, the first NL of them
+// lines) in direction dir (0 down, 1 up), NP pairs of angles from pair v0 on
+// in one pass over depth, so the depth terms are paid once for all of them.
+// One lane = one wavelength.  At each depth the lane forms, without
+// subtracting nearly equal numbers,
+//   I_eff = I - Psi* eta_active = I_u e^{-dtau} + w_u S_u + w_o eta_bg/chi,
+//   1 - Psi* chi_j = (1 - w_o) + w_o (chi - chi_j)/chi,
+// and the contributions of a pair's two rays (weight w = w_mu/2):
+//   up_j = (c_j w phi_j) I_eff,  down_j = (c_j w phi_j) R_j (E_j (1 - Psi* chi_j) + I_eff),
+//   cross_{j,j'} = c_j X_j w phi_j Psi* U_j';
+// the warp sums them over its wavelengths and gives the total of each of the
+// M = K (K + 1) values, of every pair for itself, to one lane, which hands it
+// on (out(total, value, pair, depth)).
+// Every operation's rounding is spelled out, and the pairs' totals are added
+// in the order (pair, direction).  Two reasons: c_j (1e23) meets phi_j (down
+// to 1e-18) before I_eff (1e-30 below a cold temperature minimum) does, which
+// keeps every term in the FP32 range; and a few columns in 65536 lie so near a
+// singular rate matrix that another rounding of one iteration moves the
+// iteration at which their populations fail.  The results are, to the bit,
+// those of a pass per pair and direction with each term added to a tile's one
+// accumulator, whatever the launch shape, the pairs per pass and the cache.
+// 1000 columns x 12 iterations, 82 depths, 608 wavelengths, 5 angles: 34.7 ms;
+// as scalar passes of two angles, both directions in one warp, 37.6 ms.
+// (Sums over all rays taken before the constants, with one warp reduction per
+// depth, took 20.4 ms, but lose the up-rates of columns colder than 2450 K and
+// move 12 of 65536 columns: withdrawn.  What limits this one: the
+// reductions of every pair and the moves into register pairs keep the issue
+// slots 60 % busy, and the nine tile bodies exceed the instruction cache, 12 %
+// of the stalls; with the pairs' loop rolled up there are no such stalls, but
+// more instructions, 35.7 ms.)
+template <int K, int NL, int NP, bool CACHE, typename Out>
+__device__ __forceinline__ void sweep_pairs(const DevAtom &A, const Smem<float> &s, const KParams &p, int b, int dir,
+                                            int v0, int lane, const float *phc, Out out)
+{
+    typedef Unfused<K, NL> UF;
+    const int N = p.N, nmu = A.nmu;
+    const DevTile &tl = A.tile[b];
+    LaneC<float, K> lc;
+    load_lane<float, K>(A, p, b, lane, lc);
+    int poff[NL ? NL : 1];                       // first cache element of each line slot, this direction
+#pragma unroll
+    for (int j = 0; j < NL; ++j) poff[j] = CACHE ? phi_block(nmu, N, tl.phi[j], dir, 0) : 0;
+    constexpr int M = K * (K + 1), P = Pow2<M>::v, SH = 5 - Log2<P>::v;
+    const bool writer = (lane & ((1 << SH) - 1)) == 0;
+    const int widx = lane >> SH;
+    constexpr bool RING = CACHE && NL > 0;
+    const int blk = nmu * kWarp;
+    f2 w[NP], imu[NP];                           // weights (0: the padding ray of an odd number of angles), 1/mu
+#pragma unroll
+    for (int v = 0; v < NP; ++v) {
+        const int m = 2 * (v0 + v), m2 = m + 1 < nmu ? m + 1 : m;
+        w[v] = pk(A.wm2f[m], m + 1 < nmu ? A.wm2f[m2] : 0.0f);
+        imu[v] = pk(A.imuf[m], A.imuf[m2]);
+    }
+    // line profiles of pair v at depth k, from the cache or evaluated (the same arithmetic as the cache's build)
+    auto phi_at = [&](int v, int k, f2 (&ph)[NL ? NL : 1]) {
+        const int m = 2 * (v0 + v), m2 = m + 1 < nmu ? m + 1 : m;
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if constexpr (CACHE) {
+                const float *c = phc + poff[j] + k * blk;
+                ph[j] = pk(c[phi_elem<true>(nmu, m, lane)], c[phi_elem<true>(nmu, m2, lane)]);
+            } else {
+                const float a = s.ad[lc.sub[j] * N + k], z = dir ? 1.0f : -1.0f;
+                ph[j] = pk(line_phi(lc.q[j], z * A.muf[m], s.vz[k], s.ivth[k], a, lc.pn[j], s.vtab, p.tab64),
+                           line_phi(lc.q[j], z * A.muf[m2], s.vz[k], s.ivth[k], a, lc.pn[j], s.vtab, p.tab64));
+            }
+        }
+    };
+    // opacity, emissivity, and per line Vc phi, its opacity and U
+    struct Vals {
+        f2 chi, eta, t[NL ? NL : 1], ch[NL ? NL : 1], U[NL ? NL : 1];
+    };
+    auto vals = [&](const DepthF<K> &d, const f2 (&ph)[NL ? NL : 1], auto mask_, Vals &y, bool first) {
+        constexpr int mask = decltype(mask_)::value;
+        if constexpr (NL == 0) {                 // the same for every ray
+            float chi = d.chibg;
+#pragma unroll
+            for (int j = 0; j < K; ++j)
+                chi = mask >> j & 1 ? __fadd_rn(chi, d.chc[j]) : __fmaf_rn(lc.Vc[j], d.X[j], chi);
+            y.chi = splat(chi);
+            y.eta = splat(first && UF::eta_first ? __fmaf_rn(d.chibg, d.B, d.etac) : __fadd_rn(d.etabg, d.etac));
+        } else {
+            f2 ea = splat(d.etac);
+            y.chi = splat(d.chibg);
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+                if (j < NL) {
+                    y.t[j] = vmul(splat(lc.Vc[j]), ph[j]);
+                    y.ch[j] = vmul_rn(y.t[j], splat(d.X[j]));
+                    y.U[j] = vmul(splat(lc.Uc[j]), ph[j]);
+                    ea = vfma(splat(d.nu[j]), y.U[j], ea);
+                    y.chi = mask >> j & 1 ? vadd(y.chi, y.ch[j]) : vfma(y.t[j], splat(d.X[j]), y.chi);
+                } else {
+                    y.chi = mask >> j & 1 ? vadd(y.chi, splat(d.chc[j])) : vfma(splat(lc.Vc[j]), splat(d.X[j]), y.chi);
+                }
+            }
+            y.eta = vadd(splat(d.etabg), ea);
+        }
+    };
+    // contributions of a pair at depth k, summed over the warp
+    auto rates = [&](const DepthF<K> &d, const f2 (&ph)[NL ? NL : 1], const Vals &y, f2 ichi, f2 wo, f2 omwo, f2 psi,
+                     f2 Ieff, f2 wv, int v, int k) {
+        float val[P];
+#pragma unroll
+        for (int a = M; a < P; ++a) val[a] = 0;
+        auto both = [&](f2 x, f2 z) {            // x z of the first ray + x z of the second
+            float x0, x1, z0, z1;
+            upk(x, x0, x1);
+            upk(z, z0, z1);
+            return __fmaf_rn(x1, z1, __fmul_rn(x0, z0));
+        };
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            if (!lc.isline[j]) {
-                o[j] = 0;
-            } else if constexpr (CACHE) {
-                o[j] = phc[pb[j] + k * kWarp];
-            } else {
-                const R mu = mu_of<R>(A, r >> 1);
-                o[j] = line_phi(lc.q[j], (r & 1) ? mu : -mu, s.vz[k], s.ivth[k], s.ad[lc.sub[j] * N + k], lc.pn[j],
-                                s.vtab, p.tab64);
+            f2 other = splat(d.chibg);
+            float oc = d.chibg;                  // until a line comes in, the same for both rays
+            bool vec = false;
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+                if (q == j) continue;
+                constexpr int mask = UF::other;
+                if (q < NL) {
+                    other = mask >> q & 1 ? vadd(other, y.ch[q]) : vfma(y.t[q], splat(d.X[q]), other);
+                    vec = true;
+                } else if (vec) {
+                    other = mask >> q & 1 ? vadd(other, splat(d.chc[q])) : vfma(splat(lc.Vc[q]), splat(d.X[q]), other);
+                } else {
+                    oc = mask >> q & 1 ? __fadd_rn(oc, d.chc[q]) : __fmaf_rn(lc.Vc[q], d.X[q], oc);
+                    other = splat(oc);
+                }
             }
+            const f2 f = vfma(vmul(wo, other), ichi, omwo);          // 1 - Psi* chi_j
+            f2 cw = vmul(splat(lc.c[j]), wv);
+            if (j < NL) cw = vmul(cw, ph[j < NL ? j : 0]);
+            const f2 cr = vmul(cw, splat(d.Rs[j])), cx = vmul(vmul(cw, splat(d.X[j])), psi);
+            val[j] = both(cw, Ieff);
+            val[K + j] = both(cr, vfma(splat(lc.E[j]), f, Ieff));
+#pragma unroll
+            for (int q = 0; q < K; ++q)
+                if (q != j)
+                    val[2 * K + j * (K - 1) + (q < j ? q : q - 1)] = both(cx, q < NL ? y.U[q < NL ? q : 0] : splat(d.Uct[q]));
+        }
+        const float t = reduce_scatter<P>(val, lane);
+        if (writer && widx < M) out(t, widx, v0 + v, k);
+    };
+    // boundary point: I = 0 at the top; at the bottom the diffusion condition,
+    // which needs chi and B one point up
+    const int k0 = dir == 0 ? 0 : N - 1;
+    f2 I[NP], chip[NP], Sp[NP];
+    {
+        DepthF<K> d2, d;
+        if (dir == 1) depth_f<K, NL>(s, lc, N - 2, N, d2);
+        depth_f<K, NL>(s, lc, k0, N, d);
+#pragma unroll
+        for (int v = 0; v < NP; ++v) {
+            f2 ph[NL ? NL : 1], chi2;
+            Vals y;
+            if (dir == 1) {
+                phi_at(v, N - 2, ph);
+                vals(d2, ph, std::integral_constant<int, UF::next>(), y, false);
+                chi2 = y.chi;
+            }
+            phi_at(v, k0, ph);
+            vals(d, ph, std::integral_constant<int, UF::first>(), y, true);
+            const f2 ichi = vrcp(y.chi);
+            I[v] = splat(0.0f);
+            if (dir == 1) {
+                const int m = 2 * (v0 + v), m2 = m + 1 < nmu ? m + 1 : m;
+                const f2 g = vmul(pk(A.muf[m], A.muf[m2]), splat(__fsub_rn(d.B, d2.B)));
+                I[v] = vfma(g, vrcp(vmul(vmul(splat(0.5f), vadd(y.chi, chi2)), splat(s.dz[N - 2]))), splat(d.B));
+            }
+            chip[v] = y.chi;
+            Sp[v] = vmul(y.eta, ichi);
+            rates(d, ph, y, ichi, splat(0.0f), splat(1.0f), splat(0.0f), I[v], w[v], v, k0);
+        }
+    }
+    // profile ring: the copies of step st's depth go into slot st mod 3, issued
+    // two steps ahead (one commit group per step, empty past the end)
+    const int rstride = A.maxnl * blk, gstep = dir == 0 ? blk : -blk;
+    float *ring = nullptr;
+    const float *src = phc;                      // this lane's first element of the next depth to copy
+    int fst = 1, foff = rstride, roff = rstride; // its step, its ring offset; the offset being read
+    if constexpr (RING) {
+        ring = reinterpret_cast<float *>(warp_scratch(s, p, threadIdx.x >> 5));
+        src = phc + (dir == 0 ? 1 : N - 2) * blk + 4 * lane;
+    }
+    auto ring_fill = [&]() {
+        if constexpr (RING) {
+            if (fst < N) {
+                float *dst = ring + foff + 4 * lane;
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {   // nmu x 32 values: at most two 16-byte pieces a lane
+                    if (lane < nmu * 8) cp_async16(dst + j * blk, src + poff[j]);
+                    if (lane + kWarp < nmu * 8) cp_async16(dst + j * blk + 4 * kWarp, src + poff[j] + 4 * kWarp);
+                }
+            }
+            cp_async_commit();
+            ++fst;
+            src += gstep;
+            foff = foff == 2 * rstride ? 0 : foff + rstride;
+        }
+    };
+    ring_fill();
+    ring_fill();
+    for (int st = 1; st < N; ++st) {
+        const int k = dir == 0 ? st : N - 1 - st;
+        const float *rg = nullptr;
+        if constexpr (RING) {
+            cp_async_wait<1>();
+            __syncwarp();
+            rg = ring + roff;
+            ring_fill();   // into the slot read one step ago
+            roff = roff == 2 * rstride ? 0 : roff + rstride;
+        }
+        DepthF<K> d;
+        depth_f<K, NL>(s, lc, k, N, d);
+        const float hz = 0.5f * (dir == 0 ? s.dz[k - 1] : s.dz[k]);
+#pragma unroll
+        for (int v = 0; v < NP; ++v) {
+            f2 ph[NL ? NL : 1];
+            if constexpr (RING) {
+                const int m = 2 * (v0 + v);
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const float *r = rg + j * blk + m * kWarp;
+                    // a full pair in one read; the last pair's lone angle fills both halves
+                    if (v < NP - 1) {
+                        ph[j].u = *reinterpret_cast<const unsigned long long *>(r + 2 * lane);
+                    } else {
+                        const bool full = m + 1 < nmu;
+                        const float lo = r[full ? 2 * lane : lane], hi = full ? r[2 * lane + 1] : lo;
+                        ph[j] = pk(lo, hi);
+                    }
+                }
+            } else {
+                phi_at(v, k, ph);
+            }
+            Vals y;
+            f2 e, wu, wo, omwo;
+            vals(d, ph, std::integral_constant<int, UF::step>(), y, false);
+            const f2 ichi = vrcp(y.chi), S = vmul(y.eta, ichi);
+            vsc(p, vmul(vmul(vadd(y.chi, chip[v]), splat(hz)), imu[v]), e, wu, wo, omwo);
+            const f2 base = vfma(wu, Sp[v], vmul(I[v], e));
+            I[v] = vfma(wo, S, base);
+            chip[v] = y.chi;
+            Sp[v] = S;
+            rates(d, ph, y, ichi, wo, omwo, vmul(wo, ichi), vfma(wo, vmul(splat(d.etabg), ichi), base), w[v], v, k);
+        }
+    }
+    if constexpr (RING) {
+        cp_async_wait<0>();
+        __syncwarp();
+    }
+}
+
+// The sweep with partial redistribution (PRD) or the Bezier solver (BEZ): one
+// tile (K transitions in its union, their kinds read at run time), downward
+// and upward, one angle per pass over depth; the contributions are those of
+// sweep_pairs.
+// PRD: the tile's PRD slot emits with psi = rho phi (rho of the lane's point
+// and depth from the block's scratch), PRD lanes accumulate the angle-averaged
+// mean intensity J, and every slot also accumulates its plain rates (actual
+// intensity) cw I and cw R (E + I), for the PRD update.
+// prd_I (hybrid PRD only, else nullptr): the rays' intensities at the PRD
+// points and then their dI/drho, written here, and then the rays' rho,
+// read here.
+template <typename R, int K, bool PRD, bool BEZ>
+__device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &p, int b, R *slot, int lane,
+                             R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I, const R *phc)
+{
+    const int N = p.N;
+    const DevTile &tl = A.tile[b];
+    const int nmu = A.nmu;
+    const int pi = b * kWarp + lane;
+    LaneC<R, K> lc;
+    load_lane<R, K>(A, p, b, lane, lc);
+    // cached line profiles of the current ray at depth k for the tile's line
+    // slots (0 elsewhere)
+    int pb[K];                                     // the ray's first element of each line slot's cache rows
+    auto load_ph = [&](int k, R (&o)[K]) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            if (!lc.isline[j]) o[j] = 0;
+            else o[j] = phc[pb[j] + k * kWarp];
         }
     };
     constexpr int M = K * (K + 1);
@@ -1110,34 +1279,11 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
         hyb = prd_I != nullptr && pp >= 0;
     }
 
-    // rate contributions of one ray at one depth point (add: accumulate into val)
-    auto contrib = [&](const DepthC<R, K> &d, const R (&phi)[K], const R (&chj)[K], const R (&U)[K], R ichi, R wo,
-                       R omwo, R psi, R Ieff, R wm2, R (&val)[P], bool add) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            R other = d.chibg;
-#pragma unroll
-            for (int j2 = 0; j2 < K; ++j2)
-                if (j2 != j) other += chj[j2];
-            const R f = omwo + wo * other * ichi;          // 1 - Psi* chi_j
-            const R cw = lc.c[j] * wm2 * phi[j];
-            const R v0 = cw * Ieff, v1 = cw * d.Rs[j] * (lc.E[j] * f + Ieff);
-            val[j] = add ? val[j] + v0 : v0;
-            val[K + j] = add ? val[K + j] + v1 : v1;
-            const R cx = cw * d.Xs[j] * psi;
-#pragma unroll
-            for (int j2 = 0; j2 < K; ++j2)
-                if (j2 != j) {
-                    const int a = 2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1);
-                    val[a] = add ? val[a] + cx * U[j2] : cx * U[j2];
-                }
-        }
-    };
     // contributions of one depth point to the tile's accumulators
     auto emit = [&](int k, const DepthC<R, K> &d, const R (&phi)[K], const R (&chj)[K], const R (&U)[K], R ichi,
                     R wo, R omwo, R psi, R Ieff, R Ik, R wm2, int ray) {
         R val[P];
-        contrib(d, phi, chj, U, ichi, wo, omwo, psi, Ieff, wm2, val, false);
+        ray_rates<R, K, P>(lc, d, phi, chj, U, ichi, wo, omwo, psi, Ieff, wm2, val, false);
         if constexpr (PRD) {
 #pragma unroll
             for (int j = 0; j < K; ++j) {
@@ -1181,7 +1327,7 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
             const int ray = 2 * m + dir;
 #pragma unroll
             for (int j = 0; j < K; ++j)
-                pb[j] = CACHE && lc.isline[j] ? phi_ray(nmu, N, tl.phi[j], dir, m) + lane : 0;
+                pb[j] = lc.isline[j] ? phi_ray(nmu, N, tl.phi[j], dir, m) + lane : 0;
             R I, chip = 0, Sp;
             // rho of the lane's PRD point: the static-frame ratio, or (hybrid)
             // this ray's interpolated gas-frame ratio
@@ -1197,13 +1343,13 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
                     depth_consts<R, K, PRD>(s, lc, N - 2, N, d2, rl ? rl[N - 2] : (R)1, tl.prd_slot);
                     B2 = d2.B;
                     R phi[K], chj[K], U[K], eta;
-                    load_ph(N - 2, ray, pc);
+                    load_ph(N - 2, pc);
                     angle_vals<R, K, PRD>(lc, d2, pc, chip, eta, phi, chj, U);
                 }
                 DepthC<R, K> d;
                 depth_consts<R, K, PRD>(s, lc, k0, N, d, rl ? rl[k0] : (R)1, tl.prd_slot);
                 R chi, eta, phi[K], chj[K], U[K];
-                load_ph(k0, ray, pc);
+                load_ph(k0, pc);
                 angle_vals<R, K, PRD>(lc, d, pc, chi, eta, phi, chj, U);
                 const R ichi = rcp<R>(chi);
                 if (dir == 0) {
@@ -1220,14 +1366,14 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
             R rho_nx = (PRD && rl) ? rl[dir == 0 ? 1 : N - 2] : (R)1;
             // cached profiles, like rho, loaded one depth step ahead
             R pa[K];
-            load_ph(dir == 0 ? 1 : N - 2, ray, pa);
+            load_ph(dir == 0 ? 1 : N - 2, pa);
             for (int step = 1; step < N; ++step) {
                 const int k = dir == 0 ? step : N - 1 - step;
                 const bool has_d = step + 1 < N;   // a downwind point
                 const R rho_k = rho_nx;
                 if (PRD && rl && has_d) rho_nx = rl[dir == 0 ? step + 1 : N - 2 - step];
                 R na[K];
-                load_ph(has_d ? (dir == 0 ? k + 1 : k - 1) : k, ray, na);
+                load_ph(has_d ? (dir == 0 ? k + 1 : k - 1) : k, na);
                 // quadratic Bezier step: the downwind point's opacity and source
                 // function first (its profiles and rho are the ones loaded for
                 // the next step), so that its depth terms are dead before the
@@ -1277,40 +1423,68 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
     }
 }
 
-// Work item q of the sweep: a tile, whose rays add to its accumulators one
-// after the other.  The tile's kinds are read at run time: known at compile
-// time, and with the two directions as separate items, the Bezier solver takes
-// 21.0 instead of 24.9 ms (300 columns x 8 iterations), but the contributions
-// then round and add up in another order, and 8 of 65536 columns, whose rate
-// matrices are nearly singular, fail at another iteration.  (The nine tile
-// bodies of the PRD kernels cost more in instruction fetches than they save,
-// 3.2 -> 4.8 ms an iteration of 304 columns.)
-template <typename R, bool PRD, bool CACHE, bool BEZ>
-__device__ __forceinline__ void sweep_tile(const DevAtom &A, const Smem<R> &s, const KParams &p, int item, int lane,
-                                           R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I,
-                                           const R *phc)
+// The warps' totals of the FP32 linear sweep (with the profile cache), behind
+// the block's profiles: [pair][direction][depth][accumulator].  Kept apart, the
+// tiles' directions are independent work items (20 tiles on 8 warps: 5 rounds
+// of one direction instead of 3 of both) and all angles go in one pass, and
+// still the sum is taken in the order of a pass per pair and direction.
+__device__ __forceinline__ float *pair_sums(const DevAtom &A, const KParams &p, float *phc)
 {
-    const int b = A.order[item];
-    const DevTile &tl = A.tile[b];
-    R *slot = s.slot + (size_t)tl.acc_off * p.N;
-    switch (tl.K) {
-    case 1: sweep_tile_k<R, 1, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
-    case 2: sweep_tile_k<R, 2, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
-    default: sweep_tile_k<R, 3, PRD, CACHE, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+    return phc + (size_t)A.nphi * 2 * A.nmu * p.N * kWarp;
+}
+__device__ __forceinline__ void sum_pairs(const DevAtom &A, const KParams &p, const float *g, float *slot)
+{
+    const int n = A.macc * p.N, nq = (A.nmu + 1) / 2 * 2;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        float s = g[i];
+#pragma unroll 4
+        for (int q = 1; q < nq; ++q) s = __fadd_rn(s, g[(size_t)q * n + i]);
+        slot[i % A.macc * p.N + i / A.macc] = s;
     }
 }
 
-// work item q of the sweep: a tile in one direction (split), or in both
-template <typename R, int NV, bool CACHE>
+// Work item q of the sweep: a tile, in one direction (split: sweep_unit and
+// the cached sweep_pairs) or in both.
+template <typename R, bool PRD, bool CACHE, bool BEZ, int NP>
 __device__ __forceinline__ void sweep_item(const DevAtom &A, const Smem<R> &s, const KParams &p, int q, int lane,
-                                           const R *phc)
+                                           R *prd_rho, R *prd_J, R *prd_D, R *prd_plain, R *prd_I, R *phc)
 {
     const int b = A.order[p.split ? q >> 1 : q];
     const DevTile &tl = A.tile[b];
-    for (int dir = p.split ? q & 1 : 0; dir < (p.split ? (q & 1) + 1 : 2); ++dir) {
-        R *slot = s.slot + (size_t)(tl.acc_off + (p.split && dir ? A.macc : 0)) * p.N;
-        const bool add = !p.split && dir;
-#define RH_TILE(K_, NL_) sweep_unit<R, K_, NL_, NV, CACHE>(A, s, p, b, dir, slot, add, lane, phc)
+    const int d0 = p.split ? q & 1 : 0, d1 = p.split ? d0 + 1 : 2;
+    R *slot = s.slot + (size_t)tl.acc_off * p.N;
+    if constexpr (PRD || BEZ) {
+        // (with the kinds at compile time the nine tile bodies of the PRD
+        // kernels cost more in instruction fetches than they save, 3.2 -> 4.8
+        // ms an iteration of 304 columns)
+        switch (tl.K) {
+        case 1: sweep_tile_k<R, 1, PRD, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+        case 2: sweep_tile_k<R, 2, PRD, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+        default: sweep_tile_k<R, 3, PRD, BEZ>(A, s, p, b, slot, lane, prd_rho, prd_J, prd_D, prd_plain, prd_I, phc); break;
+        }
+    } else {
+        auto tile = [&](auto k_, auto nl_) {
+            constexpr int K = decltype(k_)::value, NL = decltype(nl_)::value;
+            if constexpr (sizeof(R) == 8) {
+                for (int dir = d0; dir < d1; ++dir)
+                    sweep_unit<K, NL, CACHE>(A, s, p, b, dir, slot + (p.split && dir ? (size_t)A.macc * p.N : 0),
+                                             !p.split && dir, lane, phc);
+            } else if constexpr (CACHE) {
+                // a pass's totals, kept apart until every unit is done (sum_pairs)
+                float *g = pair_sums(A, p, phc) + tl.acc_off;
+                for (int v0 = 0; 2 * v0 < A.nmu; v0 += NP)
+                    sweep_pairs<K, NL, NP, CACHE>(A, s, p, b, d0, v0, lane, phc, [&](float t, int a, int v, int k) {
+                        g[((size_t)(2 * v + d0) * p.N + k) * A.macc + a] = t;
+                    });
+            } else {
+                for (int v0 = 0; 2 * v0 < A.nmu; ++v0)
+                    for (int dir = 0; dir < 2; ++dir)
+                        sweep_pairs<K, NL, 1, CACHE>(A, s, p, b, dir, v0, lane, phc, [&](float t, int a, int, int k) {
+                            slot[a * p.N + k] = __fadd_rn(slot[a * p.N + k], t);   // zeroed before the sweep
+                        });
+            }
+        };
+#define RH_TILE(K_, NL_) tile(std::integral_constant<int, K_>(), std::integral_constant<int, NL_>())
         switch (tl.K * 4 + tl.nl) {
         case 4: RH_TILE(1, 0); break;
         case 5: RH_TILE(1, 1); break;
@@ -1431,7 +1605,7 @@ __device__ void hybrid_JD(const DevAtom &A, const PrdScr<R> &ps, int N)
 
 // Fill the column's profile cache: warps take (row, direction, quarter of the
 // depths), lanes their wavelengths (the same arithmetic as the uncached sweep).
-template <typename R, bool UNITS, bool PAIRS>
+template <typename R, bool RAYS, bool PAIRS>
 __device__ void build_profiles(const DevAtom &A, const Smem<R> &s, const KParams &p, R *phc)
 {
     const int N = p.N, nmu = A.nmu;
@@ -1445,21 +1619,17 @@ __device__ void build_profiles(const DevAtom &A, const Smem<R> &s, const KParams
         const R pn = lt[(RH_NLANEF * j + 5) * p.npad + pi];
         const R *ad = s.ad + (size_t)A.tr[A.tile[b].t[j]].sub * N;
         for (int k = N * part / 4; k < N * (part + 1) / 4; ++k) {
-            R *o = phc + phi_block<R>(nmu, N, row, dir, k);
+            R *o = phc + (RAYS ? phi_ray(nmu, N, row, dir, 0) + k * kWarp + lane : phi_block(nmu, N, row, dir, k));
             const R vz = s.vz[k], iv = s.ivth[k], a = ad[k];
             auto at = [&](int m) {
                 const R mu = mu_of<R>(A, m);
                 return line_phi(q, dir ? mu : -mu, vz, iv, a, pn, s.vtab, p.tab64);
             };
             int m = 0;
-            if (!UNITS)
-                for (; m < nmu; ++m) phc[phi_ray(nmu, N, row, dir, m) + k * kWarp + lane] = at(m);
-            if (PAIRS)
-                for (; m + 1 < nmu; m += 2) {
-                    const float2 v = make_float2(at(m), at(m + 1));
-                    *reinterpret_cast<float2 *>(o + phi_elem<PAIRS>(nmu, m, lane)) = v;
-                }
-            for (; m < nmu; ++m) o[phi_elem<PAIRS>(nmu, m, lane)] = at(m);
+            if constexpr (PAIRS)
+                for (; m + 1 < nmu; m += 2)
+                    *reinterpret_cast<float2 *>(o + phi_elem<PAIRS>(nmu, m, lane)) = make_float2(at(m), at(m + 1));
+            for (; m < nmu; ++m) o[RAYS ? m * N * kWarp : phi_elem<PAIRS>(nmu, m, lane)] = at(m);
         }
     }
 }
@@ -1638,16 +1808,17 @@ __device__ __forceinline__ int solve_depth(const DevAtom &A, const R *slot, int 
 // CACHE: line profiles from the per-block cache (p.phic, nullptr only for an
 // atom without lines); otherwise evaluated in the sweep.  BEZ: the quadratic
 // Bezier formal solver (its own instantiations, so that the linear kernels
-// keep their registers)
-// NV: vectors of rays per pass of sweep_unit (linear solver, complete
-// redistribution), -1: the kernels of sweep_tile_k.  FP32: 128 registers, two
-// resident blocks of 256 threads or one of 512.
-template <typename R, bool PRD, bool CACHE, bool BEZ, int NV>
-__global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(R) == 4 && NV < 0 ? 2 : 1) mali_kernel(const __grid_constant__ DevAtom A, const __grid_constant__ KParams p)
+// keep their registers).  FP32: 128 registers, two resident blocks of 256
+// threads, or (linear solver, complete redistribution) one of 512.
+// NP: pairs of angles per pass of sweep_pairs.
+template <typename R, bool PRD, bool CACHE, bool BEZ, int NP>
+__global__ void __launch_bounds__(sizeof(R) == 4 && !PRD && !BEZ ? 512 : 256, sizeof(R) == 4 && (PRD || BEZ) ? 2 : 1) mali_kernel(const __grid_constant__ DevAtom A, const __grid_constant__ KParams p)
 {
     extern __shared__ __align__(16) char smem_raw[];
     const int N = p.N, L = A.nlev;
-    constexpr bool UNITS = NV >= 0;
+    constexpr bool RAYS = PRD || BEZ;                        // sweep_tile_k, which adds to its accumulators
+    constexpr bool UNITS = sizeof(R) == 8 && !RAYS;          // sweep_unit, which writes them
+    constexpr bool SUMS = sizeof(R) == 4 && !RAYS && CACHE;  // sweep_pairs, totals kept apart
     Smem<R> s = carve<R>(smem_raw, L, N, 0, A.ncont, A.nline, p.slot_rows, 0);
     const int tid = threadIdx.x, lane = tid & 31;
     const int LN = L * N;
@@ -1703,7 +1874,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(
         const double *Cr = p.Crate + cN * 2 * A.ntr;
         if (phc) {
             __syncthreads();   // the column's Doppler widths, velocities and damping
-            build_profiles<R, UNITS, UNITS && sizeof(R) == 4>(A, s, p, phc);
+            build_profiles<R, RAYS, sizeof(R) == 4 && !RAYS>(A, s, p, phc);
         }
         if constexpr (PRD) {
             // redistribution kernels of the column: K_ij = R(x_j, x_i) w_j / sum_j (.),
@@ -1795,7 +1966,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(
         for (it = 1; it <= maxiter; ++it) {
             double fcr = crsw > 1.0 ? fmax(1.0, crsw * pow(10.0, -(double)(it - 1))) : 1.0;
             for (int i = tid; i < LN; i += blockDim.x) s.nr[i] = (R)(s.n[i] * p.inv_nref);
-            if (!UNITS)
+            if (!UNITS && !SUMS)
                 for (int i = tid; i < A.macc * N; i += blockDim.x) s.slot[i] = 0;
             if constexpr (PRD) {
                 for (int i = tid; i < A.npp * N; i += blockDim.x) {
@@ -1813,16 +1984,16 @@ __global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(
                 if (lane == 0) q = atomicAdd(&s.ibuf[1], 1);
                 q = __shfl_sync(0xffffffffu, q, 0);
                 if (q >= (p.split ? 2 * A.ntile : A.ntile)) break;
-                if constexpr (UNITS) {
-                    sweep_item<R, NV, CACHE>(A, s, p, q, lane, phc);
-                } else {
-                    sweep_tile<R, PRD, CACHE, BEZ>(A, s, p, q, lane, ps.rho, ps.J, ps.D, ps.plain,
-                                                   p.prd_hybrid ? ps.Iray : nullptr, phc);
-                }
+                sweep_item<R, PRD, CACHE, BEZ, NP>(A, s, p, q, lane, ps.rho, ps.J, ps.D, ps.plain,
+                                               p.prd_hybrid ? ps.Iray : nullptr, phc);
             }
             __syncthreads();
+            if constexpr (SUMS) {
+                sum_pairs(A, p, pair_sums(A, p, phc), s.slot);
+                __syncthreads();
+            }
             // ---- rate equations: the matrices by the whole block, then one thread per depth
-            assemble_rates<R>(A, s.slot, p.split ? s.slot + (size_t)A.macc * N : s.slot, N, Cr, fcr);
+            assemble_rates<R>(A, s.slot, UNITS && p.split ? s.slot + (size_t)A.macc * N : s.slot, N, Cr, fcr);
             int bad = 0;
             double dloc = 0.0;
             for (int k = tid; k < N; k += blockDim.x) {
@@ -2113,8 +2284,8 @@ __global__ void __launch_bounds__(sizeof(R) == 4 && NV >= 0 ? 512 : 256, sizeof(
 }  // namespace mali
 
 // the column kernels' addresses (one translation unit per family, compiled in
-// parallel); nv: vectors of rays per pass of the linear solver's FP32 sweep
-const void *mali_kernel_crd32(bool cache, int nv);
+// parallel)
+const void *mali_kernel_crd32(bool cache, int np);   // np: pairs of angles per pass
 const void *mali_kernel_crd64(bool cache);
 const void *mali_kernel_bez(int precision);
 const void *mali_kernel_prd32();

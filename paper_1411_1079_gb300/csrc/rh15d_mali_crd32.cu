@@ -3,15 +3,12 @@
 
 namespace rh {
 
-const void *mali_kernel_crd32(bool cache, int nv)
+const void *mali_kernel_crd32(bool cache, int np)
 {
     using namespace mali;
-    if (!cache)
-        return nv == 1   ? (const void *)mali_kernel<float, false, false, false, 1>
-               : nv == 2 ? (const void *)mali_kernel<float, false, false, false, 2>
-                         : (const void *)mali_kernel<float, false, false, false, 3>;
-    return nv == 1   ? (const void *)mali_kernel<float, false, true, false, 1>
-           : nv == 2 ? (const void *)mali_kernel<float, false, true, false, 2>
+    if (!cache) return (const void *)mali_kernel<float, false, false, false, 1>;
+    return np == 1   ? (const void *)mali_kernel<float, false, true, false, 1>
+           : np == 2 ? (const void *)mali_kernel<float, false, true, false, 2>
                      : (const void *)mali_kernel<float, false, true, false, 3>;
 }
 
