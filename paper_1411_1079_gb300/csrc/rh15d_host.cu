@@ -743,8 +743,10 @@ int spectrum_tables(rh_ctx *c, int64_t nlambda, const double *lambda_m, std::vec
     return RH_OK;
 }
 
-// the tables of spectrum_tables on the device, one copy into the context's
-// workspace; valid until the next call on this context
+// the tables of spectrum_tables on the device, in the context's workspace;
+// valid until the next call on this context.  The copies may still read the
+// vectors when this returns (pageable memory, which this GPU can address
+// itself): the caller keeps them until it has synchronised the stream.
 struct SpecTables {
     double *nu, *spec;
     int *nact, *act;
@@ -761,16 +763,15 @@ cudaError_t spectrum_upload(rh_ctx *c, const std::vector<double> &nu, const std:
         if (e != cudaSuccess) return e;
         c->spec_cap = n;
     }
-    std::vector<char> h(n);
-    memcpy(h.data(), nu.data(), b0);
-    memcpy(h.data() + b0, spec.data(), b1);
-    memcpy(h.data() + b0 + b1, nact.data(), b2);
-    memcpy(h.data() + b0 + b1 + b2, act.data(), b3);
     t.nu = reinterpret_cast<double *>(c->spec_d);
     t.spec = reinterpret_cast<double *>(c->spec_d + b0);
     t.nact = reinterpret_cast<int *>(c->spec_d + b0 + b1);
     t.act = reinterpret_cast<int *>(c->spec_d + b0 + b1 + b2);
-    return cudaMemcpyAsync(c->spec_d, h.data(), n, cudaMemcpyHostToDevice, c->st);   // pageable: staged on return
+    cudaError_t e = cudaMemcpyAsync(t.nu, nu.data(), b0, cudaMemcpyHostToDevice, c->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(t.spec, spec.data(), b1, cudaMemcpyHostToDevice, c->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(t.nact, nact.data(), b2, cudaMemcpyHostToDevice, c->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(t.act, act.data(), b3, cudaMemcpyHostToDevice, c->st);
+    return e;
 }
 
 __global__ void validate_kernel(int64_t ncol, int ndep, const double *z, const double *T, const double *ne,
@@ -1514,7 +1515,8 @@ int rh_emergent_spectrum(rh_ctx *c, double mu, int64_t nlambda, const double *la
                             precision, c->st);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(I_out, out_d, (size_t)c->ncol * nlambda * 8, cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
+    const cudaError_t es = cudaStreamSynchronize(c->st);   // also after an error: the copies read nu, spec, ...
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) rc = fail(c, RH_ECUDA, "rh_emergent_spectrum: %s", cudaGetErrorString(e));
     if (!on_device) dfree(out_d);
     return rc;
@@ -1562,7 +1564,8 @@ int rh_emergent_stokes(rh_ctx *c, int32_t line, double g_eff, const double *B_T,
                           c->dtab_d, c->tab64_d, out_d, precision, c->st);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(iquv_out, out_d, (size_t)c->ncol * nlambda * 4 * 8, cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
+    const cudaError_t es = cudaStreamSynchronize(c->st);   // also after an error: the copies read nu, spec, ...
+    if (e == cudaSuccess) e = es;
     int rc = RH_OK;
     if (e != cudaSuccess) rc = fail(c, RH_ECUDA, "rh_emergent_stokes: %s", cudaGetErrorString(e));
     if (!on_device) {
