@@ -2,8 +2,9 @@
 column in a thousand of a cube loses a positive population in its first iterations, and a few in 65536 lie so near
 that edge that any other rounding of the sweep's contributions, or another order of their sums, moves the iteration
 at which they fail or saves them.  OUTCOMES holds such columns -- (seed, column): (status, iterations) of
-`chromosphere_cube(nx=8192, ny=1, ndep=82, seed)` -- as the sweeps that add ray after ray (c w phi) I to a tile's
-accumulators end them (status 1: all iterations done, 2: a population not positive)."""
+`chromosphere_cube(nx=8192, ny=1, ndep=82, seed)` (4096 columns with partial redistribution) -- as the sweeps that add
+ray after ray (c w phi) I to a tile's accumulators end them, with R_II-A integrated term by term (status 1: all
+iterations done, 2: a population not positive)."""
 import numpy as np
 import pytest
 
@@ -16,6 +17,9 @@ LINEAR = {(100, 5310): (2, 9), (101, 1553): (2, 5), (103, 130): (2, 7), (104, 42
           (106, 5066): (1, 12)}
 BEZIER = {(100, 3994): (2, 6), (101, 1985): (1, 8), (103, 5184): (2, 6), (104, 8125): (2, 6), (106, 3648): (1, 8),
           (106, 7772): (2, 2), (107, 1628): (1, 8), (107, 3834): (2, 2)}
+PRD = {(301, 1207): (1, 8), (301, 3232): (1, 8), (305, 3136): (1, 8)}
+HYBRID = {(301, 1847): (1, 8), (303, 2398): (1, 8), (303, 2474): (1, 8), (303, 3128): (2, 6), (303, 3745): (2, 6),
+          (304, 4066): (1, 8)}
 
 
 def _context(rh, atom, cols):
@@ -32,15 +36,22 @@ def rh():
     return m
 
 
-@pytest.mark.parametrize("formal,maxiter,outcomes", [(0, 12, LINEAR), (1, 8, BEZIER)])
-def test_nearly_singular_columns_end_as_recorded(rh, formal, maxiter, outcomes):
+CRD_ATOM = rh_synth.hydrogen_like_atom()
+PRD_ATOM = rh_synth.hydrogen_like_atom(prd_lines=((1, 2), (1, 3)), prd_nlambda=64)
+
+
+@pytest.mark.parametrize("atom,ncol,kw,outcomes", [
+    (CRD_ATOM, 8192, dict(formal=0, maxiter=12), LINEAR), (CRD_ATOM, 8192, dict(formal=1, maxiter=8), BEZIER),
+    (PRD_ATOM, 4096, dict(maxiter=8, prd_eps0=0.05, prd_hybrid=0), PRD),
+    (PRD_ATOM, 4096, dict(maxiter=8, prd_eps0=0.05, prd_hybrid=1), HYBRID)], ids=["linear", "bezier", "prd", "hybrid"])
+def test_nearly_singular_columns_end_as_recorded(rh, atom, ncol, kw, outcomes):
     parts = []
     for seed in sorted({s for s, _ in outcomes}):
-        cube = rh_synth.chromosphere_cube(nx=8192, ny=1, ndep=82, seed=seed)
+        cube = rh_synth.chromosphere_cube(nx=ncol, ny=1, ndep=82, seed=seed)
         parts.append(rh_synth.subset(cube, [c for s, c in sorted(outcomes) if s == seed]))
     cols = {k: np.concatenate([p[k] for p in parts]) for k in parts[0]}
-    ctx = _context(rh, rh_synth.hydrogen_like_atom(), cols)
-    ctx.iterate(maxiter=maxiter, tol=0.0, precision=1, formal=formal)
+    ctx = _context(rh, atom, cols)
+    ctx.iterate(tol=0.0, precision=1, **kw)
     _, iters, status, _ = ctx.populations()
     got = {k: (int(status[i]), int(iters[i])) for i, k in enumerate(sorted(outcomes))}
     assert got == outcomes
