@@ -1942,9 +1942,9 @@ int rh_solve(rh_ctx *c, const rh_solve_opts *o, rh_solve_stats *st)
     }
     set_prd(c, base, o->pass1.prd_eps0, o->pass1.prd_hybrid);
     set_phic(c, base);
-    const int bw_used = base.block_warps > 0 ? base.block_warps : (prec ? 8 : 4);
-    const int ctas_max = mali_max_ctas_per_sm(c->da, c->ndep, prec, bw_used);
-    const int ctas_used = base.ctas_per_sm > 0 ? std::min(base.ctas_per_sm, ctas_max) : ctas_max;
+    base.nwork = c->ncol;
+    int bw_used = 0, ctas_used = 0;
+    mali_launch_shape(c->da, c->ndep, base, &bw_used, &ctas_used);
 
     char eb[256] = {0};
     int replayed = 0, nkern = 0;

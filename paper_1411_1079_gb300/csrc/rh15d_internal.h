@@ -659,6 +659,7 @@ size_t mali_nghist_bytes_per_block(const DevAtom &A, int ndep);
 int mali_smem_layout(int precision, int L, int N, int ntr, int ncont, int nline, int macc, int ring_warps,
                      size_t *offsets, int noff, size_t *bytes);
 int mali_max_ctas_per_sm(const DevAtom &A, int ndep, int precision, int block_warps);
+void mali_launch_shape(const DevAtom &A, int ndep, const IterLaunch &o, int *warps, int *ctas);
 size_t mali_prd_bytes_per_block(const DevAtom &A, int ndep, int precision);
 size_t mali_phic_bytes_per_block(const DevAtom &A, int ndep, int precision);
 cudaError_t launch_mali_prealloc(const DevAtom &A, const ColumnArrays &c, const void *lane_tab, int npad,

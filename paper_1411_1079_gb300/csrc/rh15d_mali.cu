@@ -103,6 +103,20 @@ int default_warps(const DevAtom &A, const IterLaunch &o, bool bez)
     return o.precision == 1 && !o.nwork_d && o.nwork <= o.nsm ? 16 : 8;
 }
 
+// The warps, kernel and layout a launch takes: the caller's warps, or the
+// default, halved (to 4 at least) until a column fits the block's shared
+// memory (many depths, angles or overlapping lines: fewer warps' scratch).
+cudaError_t pick_shape(const DevAtom &A, int N, const IterLaunch &o, bool cache, bool bez, int &bw, Shape &s)
+{
+    bw = default_warps(A, o, bez);
+    for (;;) {
+        s = Shape();
+        const cudaError_t e = shape_of(A, N, o.precision, cache, bez, bw, s);
+        if (e != cudaSuccess || s.per_sm > 0 || o.block_warps > 0 || bw <= 4) return e;
+        bw /= 2;
+    }
+}
+
 void fill_k2(KParams &p)
 {
     // 1, -1; w_o / d and (1 - e^{-d}) / d as polynomials in d (sc_weights)
@@ -198,6 +212,15 @@ int mali_max_ctas_per_sm(const DevAtom &A, int ndep, int precision, int block_wa
     return shape_of(A, ndep, precision, true, false, block_warps, s) == cudaSuccess ? s.per_sm : 0;
 }
 
+// warps per block and resident blocks per SM of a launch with the profile cache
+void mali_launch_shape(const DevAtom &A, int ndep, const IterLaunch &o, int *warps, int *ctas)
+{
+    Shape s;
+    *warps = *ctas = 0;
+    if (pick_shape(A, ndep, o, true, o.formal == 1, *warps, s) != cudaSuccess) return;
+    *ctas = o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, s.per_sm) : s.per_sm;
+}
+
 cudaError_t launch_mali(const DevAtom &A, const ColumnArrays &c, const void *lane_tab, int npad, const float4 *vtab,
                         double nref, double *nghist, size_t nghist_cap, int *queue, const IterLaunch &o,
                         cudaStream_t st, float *ms_out, int *grid_out, char *err, size_t errn)
@@ -239,14 +262,9 @@ cudaError_t launch_mali_prealloc(const DevAtom &A, const ColumnArrays &c, const 
         snprintf(err, errn, "the Bezier formal solver needs the profile cache (an earlier rh_iterate or rh_solve)");
         return cudaErrorInvalidValue;
     }
-    int bw = default_warps(A, o, bez);
+    int bw = 0;
     Shape s;
-    cudaError_t e = shape_of(A, p.N, o.precision, cache, bez, bw, s);
-    if (e == cudaSuccess && s.per_sm < 1 && o.block_warps <= 0 && bw > 4) {   // many depths: fewer warps' scratch
-        bw = 4;
-        s = Shape();
-        e = shape_of(A, p.N, o.precision, cache, bez, bw, s);
-    }
+    cudaError_t e = pick_shape(A, p.N, o, cache, bez, bw, s);
     if (e != cudaSuccess) return e;
     if (s.per_sm < 1) {
         snprintf(err, errn, "column kernel does not fit: %zu B shared memory, %d threads", s.sm, bw * kWarp);
