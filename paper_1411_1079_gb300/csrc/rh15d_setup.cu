@@ -91,15 +91,16 @@ __global__ void lte_setup_kernel(const __grid_constant__ DevAtom A, ColumnArrays
 // short-characteristics sweep from the diffusion condition at the bottom,
 // FP64 opacities, the sweep in R.
 //
-// A block owns one column and lc of its wavelengths.  What depends on depth
+// A block owns one column and lc of its wavelengths, or all (lc) wavelengths of
+// cpb columns where those are fewer than a warp.  What depends on depth
 // only (h/kT, background coefficients, Doppler width, path lengths,
 // populations, continuum ratios, damping of the lines in use) is formed once
 // into shared memory, kw depths at a time; then a thread walks the depths of
 // its wavelength.  The kernel is bound by the FP64 pipe, so the table-driven
 // functions of rh15d_math64.h carry the points: one exponential, the Voigt
 // function of the active lines, one exponential or one polynomial of the
-// step.  4096 columns x 82 depths x 201 wavelengths, FP64: rh_emergent_spectrum 229 -> 32 ms
-// (about 300 FP64 instructions a point at the FP64 pipe's rate).
+// step.  4096 columns x 82 depths x 201 wavelengths, FP64: rh_emergent_spectrum 229 -> 24.6 ms
+// (about 230 FP64 instructions a point at the FP64 pipe's rate).
 // The sweep over a segment of depths is the map I -> A I + B, so with few
 // columns a wavelength's depths are split over G threads, whose maps are
 // composed at the end (all terms positive: no cancellation); each segment
@@ -111,17 +112,18 @@ template <typename R>
 __global__ void __launch_bounds__(kSpecThreads, 2)
     spectrum_kernel(const __grid_constant__ DevAtom A, ColumnArrays c, double mu, int64_t nlam, const double *nu_d,
                     const int *nact_d, const int *act_d, const double *spec, const double *tab_g, unsigned lines,
-                    int lc, int G, int kw, double *out)
+                    int lc, int G, int kw, int cpb, double *out)
 {
     extern __shared__ double sx[];
     __shared__ R comb[2][kSpecThreads];
-    double *tab = sx, *fld = sx + kT64Size, *pop = fld + XF_N * kw, *gc = pop + A.nlev * kw, *da = gc + A.ncont * kw;
+    const int W = cpb * kw;                        // entries of a table: kw depths of each column
+    double *tab = sx, *fld = sx + kT64Size, *pop = fld + XF_N * W, *gc = pop + A.nlev * W, *da = gc + A.ncont * W;
     const int nchunk = (int)((nlam + lc - 1) / lc), N = c.ndep, L = A.nlev;
-    const int64_t col = blockIdx.x / nchunk;
-    const int g = threadIdx.x / lc;
+    const int64_t col0 = (int64_t)(blockIdx.x / nchunk) * cpb;
+    const int part = threadIdx.x / lc, g = cpb > 1 ? 0 : part, ci = cpb > 1 ? part : 0;
+    const int64_t col = col0 + ci;
     const int64_t j = (int64_t)(blockIdx.x % nchunk) * lc + threadIdx.x % lc;
-    const bool on = j < nlam;
-    const size_t cN = (size_t)col * N;
+    const bool on = j < nlam && ci < cpb && col < c.ncol;
     const double e2 = kQ * kQ / (4.0 * kPi * kEps0);
     const double Cff = e2 * e2 * e2 * 4.0 / (3.0 * kMe * kH * kC) * sqrt(2.0 * kPi / (3.0 * kK * kMe));
     for (int i = threadIdx.x; i < kT64Size; i += blockDim.x) tab[i] = tab_g[i];
@@ -135,37 +137,40 @@ __global__ void __launch_bounds__(kSpecThreads, 2)
     double Bp = 0;
     for (int w0 = 0; w0 < N; w0 += kw) {
         if (w0) __syncthreads();
-        for (int i = threadIdx.x; i < kw && w0 + i < N; i += blockDim.x) {
-            const int k = N - 1 - w0 - i;
+        for (int i = threadIdx.x; i < W; i += blockDim.x) {
+            const int ic = i / kw, k = N - 1 - w0 - (i - ic * kw);
+            if (k < 0 || col0 + ic >= c.ncol) continue;
+            const int64_t col = col0 + ic;
+            const size_t cN = (size_t)col * N;
             const double T = c.T[cN + k], ne = c.ne[cN + k], ikT = 1.0 / (kK * T);
             const double r3 = kH * kH / (2.0 * kPi * kMe) * ikT;
-            fld[XF_KT * kw + i] = kK * T;
-            fld[XF_IKT * kw + i] = ikT;
-            fld[XF_KFF * kw + i] = Cff * ne * c.np[cN + k] / sqrt(T);
-            fld[XF_NHM * kw + i] = 0.25 * c.nstar[((size_t)col * L + 0) * N + k] * ne * (r3 * sqrt(r3)) *
+            fld[XF_KT * W + i] = kK * T;
+            fld[XF_IKT * W + i] = ikT;
+            fld[XF_KFF * W + i] = Cff * ne * c.np[cN + k] / sqrt(T);
+            fld[XF_NHM * W + i] = 0.25 * c.nstar[((size_t)col * L + 0) * N + k] * ne * (r3 * sqrt(r3)) *
                                    exp(0.754 * kQ * ikT);
-            fld[XF_THOM * kw + i] = kSigmaT * ne;
+            fld[XF_THOM * W + i] = kSigmaT * ne;
             const double vth = sqrt(2.0 * kK * T / A.mass);
-            fld[XF_VTH * kw + i] = vth;
-            fld[XF_IVTH * kw + i] = 1.0 / vth;
-            fld[XF_VZ * kw + i] = mu * c.vz[cN + k];
-            fld[XF_HZ * kw + i] = k < N - 1 ? 0.5 * fabs(c.z[cN + k] - c.z[cN + k + 1]) / mu : 0.0;
-            for (int l = 0; l < L; ++l) pop[l * kw + i] = c.pops[((size_t)col * L + l) * N + k];
+            fld[XF_VTH * W + i] = vth;
+            fld[XF_IVTH * W + i] = 1.0 / vth;
+            fld[XF_VZ * W + i] = mu * c.vz[cN + k];
+            fld[XF_HZ * W + i] = k < N - 1 ? 0.5 * fabs(c.z[cN + k] - c.z[cN + k + 1]) / mu : 0.0;
+            for (int l = 0; l < L; ++l) pop[l * W + i] = c.pops[((size_t)col * L + l) * N + k];
             const double sk = N > 1 ? (double)k / (N - 1) : 0.0;
             for (int t = 0; t < A.ntr; ++t) {
                 const DevTrans &tr = A.tr[t];
                 if (!(lines >> t & 1)) continue;
                 if (tr.kind == 0)
-                    da[tr.sub * kw + i] = exp((1.0 - sk) * tr.ln_atop + sk * tr.ln_abot);
+                    da[tr.sub * W + i] = exp((1.0 - sk) * tr.ln_atop + sk * tr.ln_abot);
                 else
-                    gc[tr.sub * kw + i] = c.nstar[((size_t)col * L + tr.l) * N + k] /
+                    gc[tr.sub * W + i] = c.nstar[((size_t)col * L + tr.l) * N + k] /
                                           c.nstar[((size_t)col * L + tr.u) * N + k];
             }
         }
         __syncthreads();
         for (int s = max(sb, w0); s < min(s1, w0 + kw) && on; ++s) {
-            const int i = s - w0;
-            const double x = div64(hnu, fld[XF_KT * kw + i], fld[XF_IKT * kw + i]);
+            const int i = ci * kw + s - w0;
+            const double x = div64(hnu, fld[XF_KT * W + i], fld[XF_IKT * W + i]);
             double ex, om;
             if (x < 0.5) {   // 1 - e^{-x} by expm1 where it would cancel
                 om = -expm1(-x);
@@ -174,31 +179,31 @@ __global__ void __launch_bounds__(kSpecThreads, 2)
                 ex = exp64(-x, tab);
                 om = 1.0 - ex;
             }
-            double chi = fma(fma(fld[XF_NHM * kw + i], hm, fld[XF_KFF * kw + i] * inu3), om, fld[XF_THOM * kw + i]);
+            double chi = fma(fma(fld[XF_NHM * W + i], hm, fld[XF_KFF * W + i] * inu3), om, fld[XF_THOM * W + i]);
             const double B = tw * ex * rcp64(om);
             double eta = chi * B;
             for (int a = 0; a < na; ++a) {
                 const int t = act_d[j * RH_SPEC_ACT + a];
                 const DevTrans &tr = A.tr[t];
                 const double *f = spec + ((size_t)j * RH_SPEC_ACT + a) * RH_SPEC_F;
-                const double nl = pop[tr.l * kw + i], nup = pop[tr.u * kw + i];
+                const double nl = pop[tr.l * W + i], nup = pop[tr.u * W + i];
                 if (tr.kind == 0) {
-                    const double ivth = fld[XF_IVTH * kw + i];
+                    const double ivth = fld[XF_IVTH * W + i];
                     double H, Ld;
-                    voigt64<false>(da[tr.sub * kw + i], div64(f[3] - fld[XF_VZ * kw + i], fld[XF_VTH * kw + i], ivth), tab,
+                    voigt64<false>(da[tr.sub * W + i], div64(f[3] - fld[XF_VZ * W + i], fld[XF_VTH * W + i], ivth), tab,
                                    H, Ld);
                     const double ph = (R)H * (f[4] * ivth);
                     chi = fma(f[0] * ph, fma(-f[2], nup, nl), chi);
                     eta = fma(f[1] * ph, nup, eta);
                 } else {
-                    const double Ge = gc[tr.sub * kw + i] * ex;
+                    const double Ge = gc[tr.sub * W + i] * ex;
                     chi = fma(f[0], fma(-Ge, nup, nl), chi);
                     eta = fma(f[1] * Ge, nup, eta);
                 }
             }
             const R chiR = (R)chi, S = (R)(eta * rcp64(chi));
             if (s > sb) {
-                const R hz = (R)fld[XF_HZ * kw + i], sum = chiR + chip;
+                const R hz = (R)fld[XF_HZ * W + i], sum = chiR + chip;
                 if (s == 1)   // the bottom point's intensity: diffusion approximation
                     Bm = (R)Bp + (R)mu * ((R)Bp - (R)B) / (sum * hz * (R)mu), Am = 0;
                 R e, wu, wo;
@@ -910,7 +915,7 @@ cudaError_t launch_spectrum(const DevAtom &A, const ColumnArrays &c, double mu, 
     const int N = c.ndep;
     // depths per shared-memory table: all of them, or what 64 KB hold
     const size_t per_k = sizeof(double) * (size_t)(XF_N + A.nlev + A.ncont + A.nline);
-    const int kw = (int)std::min<size_t>((size_t)N, 65536 / per_k);
+    int kw = (int)std::min<size_t>((size_t)N, 65536 / per_k);
     const int64_t rows = (nlam + 31) / 32;   // warps per column with one thread per wavelength
     int G = 1, lc = (int)std::min<int64_t>(kSpecThreads, 32 * rows);
     if (c.ncol * rows < 8LL * nsm && kw == N) {
@@ -919,14 +924,30 @@ cudaError_t launch_spectrum(const DevAtom &A, const ColumnArrays &c, double mu, 
         if (G > 1) lc = 32;
     }
     while (G == 1 && lc > 32 && c.ncol * ((nlam + lc - 1) / lc) < 2LL * nsm) lc -= 32;
-    const int64_t blocks = c.ncol * ((nlam + lc - 1) / lc);
+    // fewer wavelengths than a warp has lanes: several columns a block, about
+    // 128 threads and as many table entries a window, while at least four
+    // blocks an SM remain.  65536 columns x 82 depths, FP64: one continuum
+    // wavelength 24.5 (a column a block; one thread per column and wavelength
+    // without tables 4.7) -> 3.7 ms, one in H alpha 57.4 (23.6) -> 4.9, 8 there
+    // 58.0 (196) -> 14.4, 31 there 59.0 (673) -> 53.0; 1300 columns, one
+    // continuum wavelength 0.71 (1.30) -> 0.50
+    int cpb = 1;
+    if (G == 1 && nlam < 32) {
+        cpb = (int)std::max<int64_t>(1, std::min<int64_t>(128 / nlam, c.ncol / (4LL * nsm)));
+        if (cpb > 1) {
+            lc = (int)nlam;
+            kw = (int)std::min<size_t>((size_t)N, std::max<size_t>(1, 32768 / (per_k * cpb)));
+        }
+    }
+    const int64_t blocks = cpb > 1 ? (c.ncol + cpb - 1) / cpb : c.ncol * ((nlam + lc - 1) / lc);
     if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-    const size_t sm = sizeof(double) * kT64Size + per_k * kw;
+    const size_t sm = sizeof(double) * kT64Size + per_k * kw * cpb;
     auto kern = precision == 1 ? spectrum_kernel<float> : spectrum_kernel<double>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)blocks, lc * G, sm, st>>>(A, c, mu, nlam, nu_d, nact_d, act_d, spec_d, tab64, lines, lc, G, kw,
-                                               out);
+    const int threads = cpb > 1 ? (lc * cpb + 31) / 32 * 32 : lc * G;
+    kern<<<(unsigned)blocks, threads, sm, st>>>(A, c, mu, nlam, nu_d, nact_d, act_d, spec_d, tab64, lines, lc, G, kw,
+                                                cpb, out);
     return cudaGetLastError();
 }
 
