@@ -412,11 +412,13 @@ int rh_surrogate_file_info(const char *path, int32_t *sizes_out, int64_t *nparam
 /* counters, the warps' line-profile rings) and the carve's end in           */
 /* offsets_out[0..15], and the bytes the launch allocates in bytes_out (the  */
 /* same function sizes and carves, so the two are equal).  macc: rows of the  */
-/* rate accumulators per depth (twice the tiles' accumulators where a tile's */
+/* rate accumulators per depth (at least the rate-matrix entries in use, two  */
+/* rows each in FP32; in FP64 twice the tiles' accumulators where a tile's    */
 /* two directions are separate work items).  ring_warps (0..32): units of     */
 /* 2304 bytes of per-warp scratch (profile ring, ray states) that do not fit  */
 /* into the Voigt table's place, which the sweep reuses.  A launch lays out    */
-/* with no collisional-rate region (they are read from device memory).       */
+/* with no collisional-rate region (ntr = 0: they are read from device         */
+/* memory).                                                                    */
 /* RH_EINVAL for sizes outside the library's limits.                        */
 int rh_column_smem_layout(int32_t precision, int32_t nlev, int32_t ndep, int32_t ntr, int32_t ncont, int32_t nline,
                           int32_t macc, int32_t ring_warps, size_t *offsets_out, size_t *bytes_out);

@@ -786,12 +786,11 @@ __device__ void sweep_unit(const DevAtom &A, const Smem<double> &s, const KParam
     }
 }
 
-// Rate contributions of one ray at one depth point (add: accumulate into
-// val); see sweep_pairs.
+// Rate contributions of one ray at one depth point (see sweep_pairs)
 template <typename R, int K, int P>
 __device__ __forceinline__ void ray_rates(const LaneC<R, K> &lc, const DepthC<R, K> &d, const R (&phi)[K],
                                           const R (&chj)[K], const R (&U)[K], R ichi, R wo, R omwo, R psi, R Ieff,
-                                          R wm2, R (&val)[P], bool add)
+                                          R wm2, R (&val)[P])
 {
 #pragma unroll
     for (int j = 0; j < K; ++j) {
@@ -801,16 +800,12 @@ __device__ __forceinline__ void ray_rates(const LaneC<R, K> &lc, const DepthC<R,
             if (j2 != j) other += chj[j2];
         const R f = omwo + wo * other * ichi;          // 1 - Psi* chi_j
         const R cw = lc.c[j] * wm2 * phi[j];
-        const R v0 = cw * Ieff, v1 = cw * d.Rs[j] * (lc.E[j] * f + Ieff);
-        val[j] = add ? val[j] + v0 : v0;
-        val[K + j] = add ? val[K + j] + v1 : v1;
+        val[j] = cw * Ieff;
+        val[K + j] = cw * d.Rs[j] * (lc.E[j] * f + Ieff);
         const R cx = cw * d.Xs[j] * psi;
 #pragma unroll
         for (int j2 = 0; j2 < K; ++j2)
-            if (j2 != j) {
-                const int a = 2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1);
-                val[a] = add ? val[a] + cx * U[j2] : cx * U[j2];
-            }
+            if (j2 != j) val[2 * K + j * (K - 1) + (j2 < j ? j2 : j2 - 1)] = cx * U[j2];
     }
 }
 
@@ -1283,7 +1278,7 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
     auto emit = [&](int k, const DepthC<R, K> &d, const R (&phi)[K], const R (&chj)[K], const R (&U)[K], R ichi,
                     R wo, R omwo, R psi, R Ieff, R Ik, R wm2, int ray) {
         R val[P];
-        ray_rates<R, K, P>(lc, d, phi, chj, U, ichi, wo, omwo, psi, Ieff, wm2, val, false);
+        ray_rates<R, K, P>(lc, d, phi, chj, U, ichi, wo, omwo, psi, Ieff, wm2, val);
         if constexpr (PRD) {
 #pragma unroll
             for (int j = 0; j < K; ++j) {
