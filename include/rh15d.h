@@ -416,9 +416,9 @@ int rh_surrogate_file_info(const char *path, int32_t *sizes_out, int64_t *nparam
 /* rows each in FP32; in FP64 twice the tiles' accumulators where a tile's    */
 /* two directions are separate work items).  ring_warps (0..32): units of     */
 /* 2304 bytes of per-warp scratch (profile ring, ray states) that do not fit  */
-/* into the Voigt table's place, which the sweep reuses.  A launch lays out    */
-/* with no collisional-rate region (ntr = 0: they are read from device         */
-/* memory).                                                                    */
+/* into the places of the accumulators (FP32) and of the Voigt table, which   */
+/* the sweep reuses.  A launch lays out with no collisional-rate region        */
+/* (ntr = 0: they are read from device memory).                                */
 /* RH_EINVAL for sizes outside the library's limits.                        */
 int rh_column_smem_layout(int32_t precision, int32_t nlev, int32_t ndep, int32_t ntr, int32_t ncont, int32_t nline,
                           int32_t macc, int32_t ring_warps, size_t *offsets_out, size_t *bytes_out);

@@ -45,7 +45,7 @@ struct Shape {
     const void *fn = nullptr;
     size_t sm = 0;
     int per_sm = 0;      // resident blocks per SM (0: does not fit)
-    int split = 0, piece = 0, nvp = 0, slot_rows = 0;
+    int split = 0, piece = 0, nsp = 0, nvp = 0, slot_rows = 0;
 };
 
 // The kernel for the atom and options, its shared memory with bw warps and
@@ -62,16 +62,19 @@ cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool be
     const bool f32 = precision == 1, crd = !A.nprd && !bez;
     if (A.nprd) s.fn = f32 ? (bez ? mali_kernel_prd32_bez() : mali_kernel_prd32()) : mali_kernel_prd64(bez);
     else if (bez) s.fn = mali_kernel_bez(precision);
-    else if (f32) s.fn = mali_kernel_crd32(cache, A.nmu <= 2 ? 1 : (A.nmu <= 4 || A.nmu > 6 ? 2 : 3));
+    else if (f32) s.fn = mali_kernel_crd32(cache);
     else s.fn = mali_kernel_crd64(cache);
-    if (crd)   // profile ring (FP32 with the cache) or ray states (FP64) per warp
-        s.piece = f32 ? (cache ? kRingSlots * A.maxnl * A.nmu * kWarp * (int)sizeof(float) : 0)
-                      : 3 * A.nmu * kWarp * (int)sizeof(double);
-    s.nvp = s.piece ? (int)(kVtabBytes / s.piece) : 0;
-    const int extra = s.piece && bw > s.nvp ? ((bw - s.nvp) * s.piece + kScratchUnit - 1) / kScratchUnit : 0;
+    if (crd)   // ray states, and (FP32 with the cache) the profile ring, per warp
+        s.piece = f32 ? pairs_scratch(A, cache) * (int)sizeof(float) : 3 * A.nmu * kWarp * (int)sizeof(double);
     for (int split = 0; split <= (crd && !f32 ? 1 : 0); ++split) {
         // accumulators (of both directions), or the rate-matrix entries summed in their place
         const int macc = std::max(split ? 2 * A.macc : A.macc, (f32 ? 2 : 1) * A.nent);
+        // warps whose scratch lies in the accumulators' and in the Voigt table's place (warp_scratch)
+        const int slot = macc * N * (int)sizeof(float) - 16;
+        const int nsp = s.piece && f32 && cache && slot > 0 ? slot / s.piece : 0;
+        const int nvp = s.piece && !(f32 && !cache) ? (int)(kVtabBytes / s.piece) : 0;
+        const int behind = s.piece ? std::max(0, bw - nsp - nvp) : 0;
+        const int extra = (behind * s.piece + kScratchUnit - 1) / kScratchUnit;
         const size_t sm = f32 ? smem_bytes<float>(A.nlev, N, 0, A.ncont, A.nline, macc, extra)
                               : smem_bytes<double>(A.nlev, N, 0, A.ncont, A.nline, macc, extra);
         int per = 0;
@@ -87,6 +90,8 @@ cudaError_t shape_of(const DevAtom &A, int N, int precision, bool cache, bool be
         s.sm = sm;
         s.per_sm = per;
         s.split = crd && f32 ? cache : split;
+        s.nsp = nsp;
+        s.nvp = nvp;
         s.slot_rows = macc;
     }
     return cudaSuccess;
@@ -183,7 +188,7 @@ KParams make_params(const DevAtom &A, const ColumnArrays &c, const void *lane_ta
     p.prd_scr = reinterpret_cast<char *>(o.prd_scr);
     p.prd_stride = A.nprd ? (o.precision == 1 ? prd_bytes<float>(A, c.ndep) : prd_bytes<double>(A, c.ndep)) : 0;
     p.tab64 = o.tab64;
-    p.piece = p.nvp = p.split = p.slot_rows = 0;
+    p.piece = p.nsp = p.nvp = p.split = p.slot_rows = p.scr[0] = p.scr[1] = p.scr[2] = 0;
     fill_k2(p);
     p.phic_stride = o.precision == 1 ? phic_bytes<float>(A, c.ndep) : phic_bytes<double>(A, c.ndep);
     p.phic = (o.phic && p.phic_stride && p.phic_stride <= o.phic_cap) ? reinterpret_cast<char *>(o.phic) : nullptr;
@@ -273,7 +278,13 @@ cudaError_t launch_mali_prealloc(const DevAtom &A, const ColumnArrays &c, const 
     p.split = s.split;
     p.slot_rows = s.slot_rows;
     p.piece = s.piece;
+    p.nsp = s.nsp;
     p.nvp = s.nvp;
+    const SmemLayout lo = o.precision == 1 ? smem_layout<float>(A.nlev, p.N, 0, A.ncont, A.nline, s.slot_rows, 0)
+                                           : smem_layout<double>(A.nlev, p.N, 0, A.ncont, A.nline, s.slot_rows, 0);
+    p.scr[0] = (int)((lo.slot + 15) & ~(size_t)15);
+    p.scr[1] = (int)lo.vtab;
+    p.scr[2] = (int)lo.ring;
     const int64_t grid = grid_of(A, p, o, s, nghist_cap);
     if (grid < 1) {
         snprintf(err, errn, "scratch of one column (Ng history %zu B) exceeds the capacity (%zu B)",

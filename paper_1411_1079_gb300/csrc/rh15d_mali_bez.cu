@@ -6,8 +6,8 @@ namespace rh {
 const void *mali_kernel_bez(int precision)
 {
     using namespace mali;
-    return precision == 1 ? (const void *)mali_kernel<float, false, true, true, 1>
-                          : (const void *)mali_kernel<double, false, true, true, 1>;
+    return precision == 1 ? (const void *)mali_kernel<float, false, true, true>
+                          : (const void *)mali_kernel<double, false, true, true>;
 }
 
 }  // namespace rh

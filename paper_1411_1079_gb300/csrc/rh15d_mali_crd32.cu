@@ -3,13 +3,11 @@
 
 namespace rh {
 
-const void *mali_kernel_crd32(bool cache, int np)
+const void *mali_kernel_crd32(bool cache)
 {
     using namespace mali;
-    if (!cache) return (const void *)mali_kernel<float, false, false, false, 1>;
-    return np == 1   ? (const void *)mali_kernel<float, false, true, false, 1>
-           : np == 2 ? (const void *)mali_kernel<float, false, true, false, 2>
-                     : (const void *)mali_kernel<float, false, true, false, 3>;
+    return cache ? (const void *)mali_kernel<float, false, true, false>
+                 : (const void *)mali_kernel<float, false, false, false>;
 }
 
 }  // namespace rh

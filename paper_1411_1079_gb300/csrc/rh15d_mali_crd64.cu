@@ -6,8 +6,8 @@ namespace rh {
 const void *mali_kernel_crd64(bool cache)
 {
     using namespace mali;
-    return cache ? (const void *)mali_kernel<double, false, true, false, 1>
-                 : (const void *)mali_kernel<double, false, false, false, 1>;
+    return cache ? (const void *)mali_kernel<double, false, true, false>
+                 : (const void *)mali_kernel<double, false, false, false>;
 }
 
 }  // namespace rh

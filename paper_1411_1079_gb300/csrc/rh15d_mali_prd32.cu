@@ -3,6 +3,6 @@
 
 namespace rh {
 
-const void *mali_kernel_prd32() { return (const void *)mali::mali_kernel<float, true, true, false, 1>; }
+const void *mali_kernel_prd32() { return (const void *)mali::mali_kernel<float, true, true, false>; }
 
 }  // namespace rh

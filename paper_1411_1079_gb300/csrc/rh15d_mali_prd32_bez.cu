@@ -3,6 +3,6 @@
 
 namespace rh {
 
-const void *mali_kernel_prd32_bez() { return (const void *)mali::mali_kernel<float, true, true, true, 1>; }
+const void *mali_kernel_prd32_bez() { return (const void *)mali::mali_kernel<float, true, true, true>; }
 
 }  // namespace rh

@@ -6,8 +6,8 @@ namespace rh {
 const void *mali_kernel_prd64(bool bez)
 {
     using namespace mali;
-    return bez ? (const void *)mali_kernel<double, true, true, true, 1>
-               : (const void *)mali_kernel<double, true, true, false, 1>;
+    return bez ? (const void *)mali_kernel<double, true, true, true>
+               : (const void *)mali_kernel<double, true, true, false>;
 }
 
 }  // namespace rh

@@ -14,9 +14,9 @@ def rh():
     return m
 
 
-def _stats(rh, ncol, ndep, **kw):
+def _stats(rh, ncol, ndep, atom=None, **kw):
     ctx = rh.Context(0)
-    ctx.setup_atom(rh_synth.hydrogen_like_atom())
+    ctx.setup_atom(atom or rh_synth.hydrogen_like_atom())
     ctx.load_columns(rh_synth.chromosphere_cube(nx=ncol, ny=1, ndep=ndep, seed=4))
     return ctx.solve(maxiter=1, rescue=False, autotune=0, **kw)
 
@@ -29,12 +29,8 @@ def test_reported_shape_is_the_default(rh, ncol, kw, warps):
     assert s["block_warps"] == warps and s["ctas_per_sm"] >= 1
 
 
-def test_many_depths_halve_the_warps(rh):
-    seen = []
-    for ndep in range(280, 400, 4):
-        try:
-            seen.append(_stats(rh, 1, ndep, precision=1)["block_warps"])
-        except rh.RhError:      # more depths than a block's shared memory holds
-            break
-    assert seen[0] == 16 and 8 in seen
-    assert seen == sorted(seen, reverse=True)
+def test_scratch_that_does_not_fit_halves_the_warps(rh):
+    # three lines per tile and eight angles: 16 warps' profile rings fill the block at some depths, 8 warps' do not
+    atom = rh_synth.hydrogen_like_atom(qwing=1000.0, nmu=8)
+    seen = {n: _stats(rh, 1, n, atom, precision=1)["block_warps"] for n in (20, 60, 82, 100, 128, 160)}
+    assert set(seen.values()) == {16, 8}, seen
