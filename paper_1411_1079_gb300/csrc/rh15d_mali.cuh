@@ -1402,6 +1402,14 @@ __device__ void sweep_tile_k(const DevAtom &A, const Smem<R> &s, const KParams &
                 if (PRD && rl && has_d) rho_nx = rl[dir == 0 ? step + 1 : N - 2 - step];
                 R na[K];
                 load_ph(has_d ? (dir == 0 ? k + 1 : k - 1) : k, na);
+                // the profiles three depths on into L1: one step of look-ahead
+                // does not cover their HBM latency
+                if (BEZ && step + 3 < N) {
+#pragma unroll
+                    for (int j = 0; j < K; ++j)
+                        if (lc.isline[j])
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(phc + pb[j] + (dir == 0 ? k + 3 : k - 3) * kWarp));
+                }
                 // quadratic Bezier step: the downwind point's opacity and source
                 // function first (its profiles and rho are the ones loaded for
                 // the next step), so that its depth terms are dead before the
