@@ -39,21 +39,21 @@ TRAIN_SEED = 4321          # training cube (disjoint from the evaluated cube, se
 TRAIN_EPOCHS = 10
 METRIC = "converged columns/s to max|dn/n|<1e-3"
 # FP32 operations per formal-solver point (one depth x lambda x mu, both
-# sweep directions) the column kernel executes: scalar thread-level operations
-# (2 x FFMA + FADD + FMUL, predicated-on threads) counted by ncu on 608 columns
+# sweep directions) the column kernel executes, counted by ncu on 608 columns
 # x 12 iterations (about the iterations a column takes from the learned
-# guess), divided by their points (28.8), plus the packed two-angle operations,
-# which those counters leave out, counted from the sweep's source for the
-# grid's tiles (55 per ray and direction, padding ray included: 139)
-FLOP_PER_PT = 168.0
-# DRAM bytes (read + write) per column-iteration of the column kernel, from
-# an ncu capture (13.0 GB for 608 x 12): the line-profile cache read
-# back every iteration (1.57 MB), its build once per column and the column's
-# inputs and results
-DRAM_BYTES_PER_COLUMN_ITERATION = (11.740e9 + 1.263e9) / (608 * 12)
+# guess) and divided by their 1.819e9 points: scalar thread-level operations
+# (2 x 40.67e9 FFMA + 27.02e9 FADD + 79.52e9 FMUL, predicated-on threads: 103.3)
+# and packed two-ray instructions, which those counters leave out (32 threads
+# x (4 x 1.6863e9 FFMA2 + 2 x 0.6390e9 FMUL2 + 2 x 0.1423e9 FADD2): 146.2)
+FLOP_PER_PT = 249.5
+# DRAM bytes (read + write) per column-iteration of the column kernel, same
+# capture (20.3 GB for 608 x 12): the line-profile cache read back every
+# iteration (1.89 MB), the warps' totals, which mostly stay in L2, the cache's
+# build once per column and the column's inputs and results
+DRAM_BYTES_PER_COLUMN_ITERATION = (16.311e9 + 3.948e9) / (608 * 12)
 # warp instructions per column-iteration, same capture: the issue-slot view of
 # the same kernel (4 schedulers per SM, one warp instruction per cycle each)
-WARP_INST_PER_COLUMN_ITERATION = 9003685780 / (608 * 12)
+WARP_INST_PER_COLUMN_ITERATION = 15963407848 / (608 * 12)
 
 
 def algorithmic_flop_per_pt(atom, nu):
@@ -63,18 +63,17 @@ def algorithmic_flop_per_pt(atom, nu):
     counted apart), for the transitions actually active at each wavelength
     (no padding lanes, no inactive slots of a tile's union) and the
     optically thick branch of the SC weights (one exponential per step; the
-    polynomial of thin steps is an accuracy choice).  With n_l lines and n_c
-    continua active (K = n_l + n_c), per depth and direction, shared by the
-    angles of a pass (all of them):
-      depth terms (x, e^-x, 1-e^-x, chi_bg, B, eta_bg)     11 + 4 n_l + 9 n_c;
-      contributions from the rays' sums                    5 K + 3 K (K - 1)
-          (+ 2 n_c), the pair's halves added                (2 n_l + ...) sums;
-      warp reduce-scatter of P = 2^ceil(log2 K(K+1)) values  P - 1 + 5 - log2 P;
-    and per ray:
-      opacities (chi, eta)                                  4 n_l;
-      SC step (dtau, weights, I, I_eff, Psi*, S)            17;
-      sums: line 7 (+ 2 with continua, + 5 per further line), continua 6
-          together (+ 2 with lines).
+    polynomial of thin steps is an accuracy choice).  Per depth and direction,
+    with n_l lines and n_c continua active (K = n_l + n_c):
+      depth terms (x, e^-x, 1-e^-x, chi_bg, B, eta_bg)     11 + 2 n_l + 7 n_c,
+          shared by all angles;
+      opacities of a ray (chi, eta)                        1 + 6 n_l + 1 n_c;
+      SC step of a ray (dtau, weights, I, I_eff, Psi*, S)  19;
+      rate terms of a ray per active line (continuum)      10 (9) + (K - 1)
+          (+ 2 + (K - 1) cross terms when K > 1, + (2 + (K - 1)) added to the
+          first ray's in the second ray of a pair);
+      warp reduce-scatter of P = 2^ceil(log2 K(K+1)) values  P - 1 + 5 - log2 P
+          per pair of angles.
     Both directions count once per point."""
     h, c, k = 6.62607015e-34, 2.99792458e8, 1.380649e-23
     E = np.asarray(atom["E_J"])
@@ -87,7 +86,8 @@ def algorithmic_flop_per_pt(atom, nu):
         nue = (E[-1] - E[l]) / h
         ranges.append((nue, r * nue, 1))
     nmu = atom["nmu"]
-    share = 1.0 / nmu                        # what a depth and direction pays once
+    pairs = (nmu + 1) // 2
+    second = (nmu - pairs) / nmu             # rays that add to a pair's first
     tot = 0.0
     mufu = 0.0
     for f in nu:
@@ -96,12 +96,13 @@ def algorithmic_flop_per_pt(atom, nu):
         nc = act.count(1)
         K = max(nl + nc, 1)
         P = 1 << int(np.ceil(np.log2(K * (K + 1))))
-        nsum = (2 + (nc > 0)) * nl + nl * (nl - 1) // 2 + (3 if nc else 0)
-        dc = (11 + 4 * nl + 9 * nc) * share
-        fl = (5 * K + 3 * K * (K - 1) + 2 * nc + nsum + P - 1 + 5 - np.log2(P)) * share
-        ray = 4 * nl + 17 + nl * (7 + 2 * (nc > 0) + 5 * (nl - 1)) + ((6 + 2 * (nl > 0)) if nc else 0)
-        tot += 2 * (dc + fl + ray)
-        mufu += 2 * (2 * share + 3)          # e^-x, rcp(1 - e^-x); rcp(chi), e^-dtau, rcp(dtau)
+        dc = (11 + 2 * nl + 7 * nc) / nmu
+        av = 1 + 6 * nl + nc
+        st = 19
+        ct = 10 * nl + 9 * nc + K * (K - 1) + (K * (2 + (K - 1)) if K > 1 else 0) + K * (2 + (K - 1)) * second
+        fl = (P - 1 + 5 - np.log2(P)) * pairs / nmu
+        tot += 2 * (dc + av + st + ct + fl)
+        mufu += 2 * (2 / nmu + 3)            # e^-x, rcp(1 - e^-x); rcp(chi), e^-dtau, rcp(dtau)
     return tot / len(nu), mufu / len(nu)
 
 
@@ -721,8 +722,8 @@ def run_gpu(args):
                                   "branch (bench.algorithmic_flop_per_pt); plus %.1f MUFU operations" % alg_mufu,
                      "executed": {"flop_per_pt": FLOP_PER_PT, "achieved": achieved_exec,
                                   "frac": achieved_exec / peak_tflops,
-                                  "note": "FP32 operations executed (scalar: ncu, 608 columns x 12 iterations; packed: "
-                                          "from the sweep's source): padding, both SC forms of every step, inactive "
+                                  "note": "FP32 operations executed (ncu, 608 columns x 12 iterations, scalar and "
+                                          "packed): padding, both SC forms of every step, inactive "
                                           "slots of a tile's transition union, the profile build"},
                      "traffic": DRAM_BYTES_PER_COLUMN_ITERATION * iters / args.steps,
                      "traffic_note": "bytes per launch: ncu DRAM bytes per column-iteration on the "
